@@ -92,6 +92,7 @@ struct ddamg_ctx {
   float* lam32 = nullptr;
   bool have_vectors = false;
   bool lam64_gone = false;       // FP64 test vectors released by ddamg_trim (lam32 holds them)
+  bool lam32_fresh = false;      // lam32 was converted from lam64 since lam64 was last written
   bool have_coarse = false;
   bool dc_g5 = false;             // D_c assembled from D (G5-hermitian block by block), not given
   void* Dc = nullptr;
@@ -1330,9 +1331,26 @@ ddamg_status need_lam64(ddamg_ctx* h) {
 }
 // FP64 test vectors for a call that writes all of them
 ddamg_status revive_lam64(ddamg_ctx* h) {
+  h->lam32_fresh = false;
   if (!h->lam64_gone) return DDAMG_OK;
   TRY(dalloc_t(h, &h->lam64, (size_t)h->p.n_v * h->V24));
   h->lam64_gone = false;
+  return DDAMG_OK;
+}
+
+// FP32 test vectors for an FP32 R or P: converted when lam64 was written
+// since they last were.  The conversion moves 288 bytes per site and vector,
+// three times what R or P read: an FP32 P call on 24^3 x 48 with 24 vectors
+// takes 356 us without it and 1076 with it, R of 12 fields on 16^4 with 20
+// vectors 213 and 280.
+ddamg_status need_lam32(ddamg_ctx* h) {
+  if (!h->lam32) {
+    TRY(need_lam64(h));
+    TRY(dalloc_t(h, &h->lam32, (size_t)h->p.n_v * h->V24));
+  }
+  if (h->lam64_gone || h->lam32_fresh) return DDAMG_OK;
+  CK(convert_spinor<float, double>(h->g, h->lam64, h->lam32, h->p.n_v, h->st));
+  h->lam32_fresh = true;
   return DDAMG_OK;
 }
 
@@ -1341,6 +1359,7 @@ ddamg_status sync_lam32(ddamg_ctx* h) {
     if (!h->lam32) TRY(dalloc_t(h, &h->lam32, (size_t)h->p.n_v * h->V24));
     // after ddamg_trim the FP32 copy is the only one (and current)
     if (!h->lam64_gone) CK(convert_spinor<float, double>(h->g, h->lam64, h->lam32, h->p.n_v, h->st));
+    h->lam32_fresh = true;
     const int k = lam_half_kind(h);
     if (k >= 0) {
       if (!h->lam16) TRY(dalloc(h, &h->lam16, (size_t)h->p.n_v * h->V24 * 2));
@@ -1466,6 +1485,7 @@ ddamg_status coarse_iters_since(ddamg_ctx* h, int* its) {
 // place, or (ortho_fp32, an FP32-arithmetic inner solver whose R and P use
 // them in FP32) on the FP32 copy, which the FP64 copy then takes
 ddamg_status ortho_inner(ddamg_ctx* h) {
+  h->lam32_fresh = false;
   if (!inner32(h) || !h->p.ortho_fp32) {
     CK(orthonormalise(h->g, h->lam64, h->p.n_v, h->st));
     return DDAMG_OK;
@@ -1524,6 +1544,7 @@ ddamg_status setup_impl(ddamg_ctx* h) {
     TRY(ortho_inner(h));
     TRY(build_coarse_op(h));
     // lambda_i <- M lambda_i
+    h->lam32_fresh = false;
     for (int c0 = 0; c0 < n; c0 += ch) {
       const int cn = std::min(ch, n - c0);
       double* lv = h->lam64 + (size_t)c0 * h->V24;
@@ -3153,9 +3174,7 @@ ddamg_status ddamg_restrict(ddamg_handle h, int prec, int nrhs, const double* in
   if (!h->have_vectors) return fail(h, DDAMG_ESTATE, "no test vectors");
   return dispatch(h, prec, [&](auto* tag) -> ddamg_status {
     using R = std::remove_pointer_t<decltype(tag)>;
-    if (sizeof(R) == 8 || !h->lam32) TRY(need_lam64(h));
-    if (sizeof(R) == 4 && !h->lam32) TRY(dalloc_t(h, &h->lam32, (size_t)h->p.n_v * h->V24));
-    if (sizeof(R) == 4 && !h->lam64_gone) CK(convert_spinor<float, double>(h->g, h->lam64, h->lam32, h->p.n_v, h->st));
+    TRY(sizeof(R) == 8 ? need_lam64(h) : need_lam32(h));
     TRY(need_tmp(h, nrhs, 6));
     TRY(import_fields<R>(h, in, on_device, nrhs, (R*)h->tmp[0]));
     CK(restrict_inner<R>(h, (R*)h->tmp[0], (R*)h->tmp[1], nrhs));
@@ -3168,9 +3187,7 @@ ddamg_status ddamg_prolong(ddamg_handle h, int prec, int nrhs, const double* in,
   if (!h->have_vectors) return fail(h, DDAMG_ESTATE, "no test vectors");
   return dispatch(h, prec, [&](auto* tag) -> ddamg_status {
     using R = std::remove_pointer_t<decltype(tag)>;
-    if (sizeof(R) == 8 || !h->lam32) TRY(need_lam64(h));
-    if (sizeof(R) == 4 && !h->lam32) TRY(dalloc_t(h, &h->lam32, (size_t)h->p.n_v * h->V24));
-    if (sizeof(R) == 4 && !h->lam64_gone) CK(convert_spinor<float, double>(h->g, h->lam64, h->lam32, h->p.n_v, h->st));
+    TRY(sizeof(R) == 8 ? need_lam64(h) : need_lam32(h));
     TRY(need_tmp(h, nrhs, 6));
     TRY(coarse_in<R>(h, in, on_device, (size_t)nrhs * h->g.nb * h->n2, (R*)h->tmp[0]));
     CK(prolong_inner<R>(h, (R*)h->tmp[0], (R*)h->tmp[1], nrhs));

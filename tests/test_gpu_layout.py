@@ -39,3 +39,17 @@ def test_fp32_fields_in_and_out(L, block):
         assert_close(got, op.site(t(x)).numpy(), TOL32)
     s.close()
 
+
+def test_fp32_projections_follow_the_vectors():
+    """R and P in FP32 use the vectors set last, also on an FP64 handle (whose
+    FP32 copy is made for the call) and after an orthonormalisation."""
+    cfg = ((8, 8, 8, 8), (4, 4, 4, 4), 0.3, -0.2, 1.0, 4, 0)
+    for prec in (0, 1):
+        s = make(cfg, prec)
+        x = syn.gaussian_spinors(1, cfg[0], 11)
+        for seed in (1, 2):
+            s.set_test_vectors(syn.gaussian_spinors(4, cfg[0], seed))
+            for _ in range(2):
+                assert_close(s.restrict(x, 1), s.restrict(x, 0), 5 * TOL32)
+                s.orthonormalize()
+        s.close()
