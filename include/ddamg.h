@@ -79,13 +79,14 @@ typedef enum {
 /* Arithmetic of the smoother, coarse grid and projections.  The outer
  * FGMRES, its residual r = b - D x and the test-vector orthonormalisation
  * are FP64 (the orthonormalisation FP32 on request, ortho_fp32).  DDAMG_BF16 and DDAMG_FP16 compute in FP32 like
- * DDAMG_FP32 but store in that half type: the smoother's links, clover
- * blocks (A and A^-1) and spinor fields (each spinor divided by its site
- * norm, the largest magnitude of its 24 reals, kept in FP32), and the test
+ * DDAMG_FP32 but store in that half type: the smoother's links and clover
+ * blocks (A and A^-1; blocks of 64, 128, 192 or 256 sites), and the test
  * vectors that R and P read (D_c is assembled from the same rounded
- * vectors); the coarse operator and the remaining fields stay FP32.  As a
- * step precision, BF16 / FP16 select the half-storage D (ddamg_apply_D),
- * SAP (ddamg_sap) and block solve (ddamg_block_solve). */
+ * vectors); the coarse operator and all fields stay FP32.  As a
+ * step precision, BF16 / FP16 select the half-storage D (ddamg_apply_D; its
+ * spinors in half too, each divided by its site norm, the largest magnitude
+ * of its 24 reals, kept in FP32), SAP (ddamg_sap) and block solve
+ * (ddamg_block_solve). */
 typedef enum { DDAMG_FP64 = 0, DDAMG_FP32 = 1, DDAMG_BF16 = 2, DDAMG_FP16 = 3 } ddamg_precision;
 
 typedef struct {
@@ -360,10 +361,9 @@ DDAMG_API ddamg_status ddamg_get_coarse_plan(ddamg_handle h, int nrhs, ddamg_coa
  * storage; the coarse GMRES's block products for eight right-hand sides in
  * lockstep with the blocks streamed through shared memory, on the CUDA
  * cores (0) or the tensor cores (1, 3xTF32) ("coarse product"); the FP32
- * Schwarz sweep with the block's links and clover blocks staged in shared
- * memory (0) or read from global memory (1) ("SAP fp32"); the half-storage
- * Schwarz sweep with the staged block operators widened to FP32 in shared
- * memory (0) or kept in the half type (1) ("SAP bf16", "SAP fp16"); the
+ * Schwarz sweep with the block's links and clover blocks in registers and the
+ * residual carried between sweeps (0) or by the general kernel (1) ("SAP
+ * fp32"; the half-storage sweep has one form); the
  * coarse stencil of an assembled D_c (ddamg_apply_coarse) from all nine
  * blocks (0) or from the self and forward blocks, the backward ones by
  * G5-hermiticity (1) ("coarse stencil"). */

@@ -652,9 +652,8 @@ cudaError_t prolong_inner(ddamg_ctx* h, const R* xc, R* out, int nf) {
   });
 }
 
-// half storage: copies of the operators and the smoother's spinor buffers
+// half storage: copies of the operators
 ddamg_status half_operators(ddamg_ctx* h, int k);
-ddamg_status need_half_fields(ddamg_ctx* h, size_t nf);
 // f(S*) with S the half type of kind k (0 FP16, 1 BF16)
 template <class F>
 cudaError_t by_half(int k, F&& f) {
@@ -764,102 +763,83 @@ ddamg_status op_dslash(ddamg_ctx* h, int mode, const R* x, const R* b, R* y, int
 }
 
 // SAP from zero: x = S b
-// FP32 Schwarz sweeps with blocks the staged kernel takes: staged (0) or
-// general kernel (1), measured on the caller's fields the first time for a
-// problem (the smoother starts from x = 0, so a trial run leaves nothing
-// behind in x that the real run keeps)
-ddamg_status sap32_staged(ddamg_ctx* h, const float* b, float* x, int nf, bool* staged) {
-  *staged = true;
-  if (!sap_staged_ok(h->g)) return DDAMG_OK;
-  auto trial = [&](int var) -> cudaError_t {
-    cudaError_t e = cudaMemsetAsync(x, 0, nf * h->V24 * sizeof(float), h->st);
-    for (int cyc = 0; cyc < h->p.n_sap && e == cudaSuccess; ++cyc)
-      for (int c = 0; c < 2 && e == cudaSuccess; ++c)
-        e = sap_sweep<float>(h->g, c, h->p.mr_iters, cyc == 0 && c == 0, b, x, h->g32, h->A32, h->Ai32, nf,
-                             h->d_status, h->wait_sap, h->st, var == 0);
-    return e;
-  };
-  int v = 0;
-  TRY(tuned(h, "SAP fp32", lattice_key(h, "fp32", nf), 2, trial, &v));
-  *staged = v == 0;
+// n_sap cycles of the block kernel; the messages and residuals between the
+// sweeps live in the temporaries that a smoother call leaves free (2 and 3:
+// the coarse vectors of M, dead by then)
+ddamg_status sap_blocks(ddamg_ctx* h, int kind, const float* b, float* x, int nf) {
+  if (h->tmp.size() < 4 || h->tmp_fields < (size_t)nf) return fail(h, DDAMG_ESTATE, "no temporaries for the smoother");
+  bool fresh = false;            // operators written just now
+  if (kind >= 0) {
+    fresh = !h->gH[kind] || h->h_gen[kind] != h->op_gen;
+    TRY(half_operators(h, kind));
+  }
+  const void* gg = kind >= 0 ? h->gH[kind] : h->g32;
+  const void* aa = kind >= 0 ? h->AH[kind] : h->A32;
+  const void* ai = kind >= 0 ? h->AiH[kind] : h->Ai32;
+  for (int cyc = 0; cyc < h->p.n_sap; ++cyc)
+    for (int c = 0; c < 2; ++c) {
+      const bool zero = cyc == 0 && c == 0, more = cyc + 1 < h->p.n_sap;
+      SapStep s{cyc == 0, !zero, c == 0 || more, more, !(zero && fresh)};
+      addf(h, nf * flops_sap_sweep(h, zero));
+      CK(timed(h, 1, [&] {
+        return sap_block_sweep(h->g, kind, c, h->p.mr_iters, s, b, x, h->tmp[3], h->tmp[2], gg, aa, ai, nf, h->d_status,
+                               h->wait_sap, h->st);
+      }));
+    }
+  return DDAMG_OK;
+}
+// the same with the general kernel: x cleared, the residual recomputed
+template <class R>
+ddamg_status sap_general(ddamg_ctx* h, const R* b, R* x, int nf) {
+  CK(cudaMemsetAsync(x, 0, nf * h->V24 * sizeof(R), h->st));
+  for (int cyc = 0; cyc < h->p.n_sap; ++cyc)
+    for (int c = 0; c < 2; ++c) {
+      const bool zero = cyc == 0 && c == 0;
+      addf(h, nf * flops_sap_sweep(h, zero));
+      CK(timed(h, 1, [&] {
+        return sap_sweep<R>(h->g, c, h->p.mr_iters, zero, b, x, gauge_of<R>(h), clov_of<R>(h, false), clov_of<R>(h, true),
+                            nf, h->st);
+      }));
+    }
   return DDAMG_OK;
 }
 
-// half-storage Schwarz sweeps: the staged block operators widened to FP32
-// in shared memory (0) or kept in the half type (1), measured the first time
-// for a problem on the half right-hand sides already in hb (the smoother
-// starts from x = 0; the caller clears x afterwards)
-ddamg_status sap_half_widen(ddamg_ctx* h, int kind, int nf, bool* widen) {
-  *widen = true;
-  if (!sap_staged_ok(h->g)) return DDAMG_OK;
+// FP32 Schwarz sweeps of blocks that the block kernel takes: with it (0) or
+// with the general kernel (1), measured on the caller's fields the first time
+// for a problem (the smoother starts from x = 0, so a trial run leaves nothing
+// behind in x that the real run keeps)
+ddamg_status sap32_by_blocks(ddamg_ctx* h, const float* b, float* x, int nf, bool* blocks) {
+  *blocks = sap_block_ok(h->g);
+  if (!*blocks) return DDAMG_OK;
+  const double f0 = h->flops[h->fphase];
+  const uint64_t n0 = h->n_cls[1];
+  const bool timing = h->timing;
+  h->timing = false;             // trials are neither timed nor counted
   auto trial = [&](int var) -> cudaError_t {
-    cudaError_t e = cudaMemsetAsync(h->hx, 0, nf * h->V24 * 2, h->st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(h->hxn, 0, nf * h->g.V * sizeof(float), h->st);
-    for (int cyc = 0; cyc < h->p.n_sap && e == cudaSuccess; ++cyc)
-      for (int c = 0; c < 2 && e == cudaSuccess; ++c)
-        e = by_half(kind, [&](auto* tag) {
-          using S = std::remove_pointer_t<decltype(tag)>;
-          return sap_sweep_h<S>(h->g, c, h->p.mr_iters, cyc == 0 && c == 0, h->hb, h->hbn, h->hx, h->hxn,
-                                h->gH[kind], h->AH[kind], h->AiH[kind], nf, h->d_status, h->wait_sap, h->st,
-                                var == 0);
-        });
-    return e;
+    const ddamg_status s = var == 0 ? sap_blocks(h, -1, b, x, nf) : sap_general<float>(h, b, x, nf);
+    return s == DDAMG_OK ? cudaSuccess : cudaErrorUnknown;
   };
   int v = 0;
-  TRY(tuned(h, kind ? "SAP bf16" : "SAP fp16", lattice_key(h, kind ? "bf16" : "fp16", nf), 2, trial, &v));
-  *widen = v == 0;
-  return DDAMG_OK;
+  const ddamg_status s = tuned(h, "SAP fp32", lattice_key(h, "fp32", nf), 2, trial, &v);
+  h->timing = timing;
+  h->flops[h->fphase] = f0;
+  h->n_cls[1] = n0;
+  *blocks = v == 0;
+  return s;
 }
 
 template <class R>
 ddamg_status op_sap(ddamg_ctx* h, const R* b, R* x, int nf, int kind = -2) {
   if (kind == -2) kind = half_kind(h->p.precision);
   if constexpr (sizeof(R) == 4) {
-    // half storage: links, clover blocks and the smoother's b and x in the
-    // half type (FP32 arithmetic); b in and x out in FP32
-    if (kind >= 0 && sap_half_ok(h->g)) {
-      TRY(half_operators(h, kind));
-      TRY(need_half_fields(h, nf));
-      CK(by_half(kind, [&](auto* tag) {
-        using S = std::remove_pointer_t<decltype(tag)>;
-        return spinor_to_half<S>(h->g, b, h->hb, h->hbn, nf, h->st);
-      }));
-      bool widen = true;
-      TRY(sap_half_widen(h, kind, nf, &widen));
-      CK(cudaMemsetAsync(h->hx, 0, nf * h->V24 * 2, h->st));
-      CK(cudaMemsetAsync(h->hxn, 0, nf * h->g.V * sizeof(float), h->st));
-      for (int cyc = 0; cyc < h->p.n_sap; ++cyc)
-        for (int c = 0; c < 2; ++c) {
-          const bool zero = cyc == 0 && c == 0;
-          addf(h, nf * flops_sap_sweep(h, zero));
-          CK(timed(h, 1, [&] {
-            return by_half(kind, [&](auto* tag) {
-              using S = std::remove_pointer_t<decltype(tag)>;
-              return sap_sweep_h<S>(h->g, c, h->p.mr_iters, zero, h->hb, h->hbn, h->hx, h->hxn, h->gH[kind],
-                                    h->AH[kind], h->AiH[kind], nf, h->d_status, h->wait_sap, h->st, widen);
-            });
-          }));
-        }
-      CK(by_half(kind, [&](auto* tag) {
-        using S = std::remove_pointer_t<decltype(tag)>;
-        return spinor_from_half<S>(h->g, h->hx, h->hxn, x, nf, false, h->st);
-      }));
-      return DDAMG_OK;
-    }
+    // half storage: links and clover blocks in the half type (FP32 arithmetic
+    // and fields)
+    if (kind >= 0 && sap_block_ok(h->g)) return sap_blocks(h, kind, b, x, nf);
+    bool blocks = true;
+    TRY(sap32_by_blocks(h, b, x, nf, &blocks));
+    if (blocks) return sap_blocks(h, -1, b, x, nf);
   }
-  bool staged = true;
-  if constexpr (sizeof(R) == 4) TRY(sap32_staged(h, b, x, nf, &staged));
-  CK(cudaMemsetAsync(x, 0, nf * h->V24 * sizeof(R), h->st));
-  for (int cyc = 0; cyc < h->p.n_sap; ++cyc)
-    for (int c = 0; c < 2; ++c) {
-      bool zero = cyc == 0 && c == 0;
-      addf(h, nf * flops_sap_sweep(h, zero));
-      CK(timed(h, 1, [&] {
-        return sap_sweep<R>(h->g, c, h->p.mr_iters, zero, b, x, gauge_of<R>(h), clov_of<R>(h, false),
-                            clov_of<R>(h, true), nf, h->d_status, h->wait_sap, h->st, staged);
-      }));
-    }
-  return DDAMG_OK;
+  return sap_general<R>(h, b, x, nf);
 }
 
 template <class R>
@@ -1507,13 +1487,13 @@ ddamg_status setup_impl(ddamg_ctx* h) {
   if (inner32(h) && !h->lam32) TRY(dalloc_t(h, &h->lam32, (size_t)n * h->V24));
   if (lam_half_kind(h) >= 0 && !h->lam16) TRY(dalloc(h, &h->lam16, (size_t)n * h->V24 * 2));
   TRY(alloc_coarse(h));
-  if (half_kind(h->p.precision) >= 0 && sap_half_ok(h->g)) TRY(half_operators(h, half_kind(h->p.precision)));
+  if (half_kind(h->p.precision) >= 0 && sap_block_ok(h->g)) TRY(half_operators(h, half_kind(h->p.precision)));
   int ch = n;
   {
     size_t fr = 0, tot = 0;
     if (cudaMemGetInfo(&fr, &tot) == cudaSuccess) {
       cudaGetLastError();
-      const size_t per = 6 * h->V24 * sizeof(double) + 2 * h->V24 * 2 + 2 * h->g.V * sizeof(float);
+      const size_t per = 6 * h->V24 * sizeof(double);
       size_t avail = fr + h->tmp_fields * 6 * h->V24 * sizeof(double);
       if (h->p.hbm_budget) {
         const size_t left = h->p.hbm_budget > h->bytes ? h->p.hbm_budget - h->bytes : 0;
@@ -1602,10 +1582,7 @@ ddamg_status prepare_capture(ddamg_ctx* h) {
   if (!h->cap_st) CK(cudaStreamCreateWithFlags(&h->cap_st, cudaStreamNonBlocking));
   TRY(need_tmp(h, 1, 6));
   const int k = half_kind(h->p.precision);
-  if (k >= 0) {
-    TRY(half_operators(h, k));
-    TRY(need_half_fields(h, 1));
-  }
+  if (k >= 0) TRY(half_operators(h, k));
   if (inner32(h)) coarse_gmres_exact_bytes<float>(h->g, h->p.n_v, h->p.coarse_restart, 1);
   else coarse_gmres_exact_bytes<double>(h->g, h->p.n_v, h->p.coarse_restart, 1);
   // the D of the captured iterations (FP32 inner precision) is chosen now:
@@ -1616,17 +1593,8 @@ ddamg_status prepare_capture(ddamg_ctx* h) {
   }
   // and the smoother's kernel (the FP32 fields as scratch)
   if (inner32(h) && k < 0) {
-    bool staged = true;
-    TRY(sap32_staged(h, (const float*)h->fin, (float*)h->fout, 1, &staged));
-  }
-  if (k >= 0 && sap_half_ok(h->g)) {
-    CK(cudaMemsetAsync(h->fin, 0, h->V24 * sizeof(float), h->st));
-    CK(by_half(k, [&](auto* tag) {
-      using S = std::remove_pointer_t<decltype(tag)>;
-      return spinor_to_half<S>(h->g, (const float*)h->fin, h->hb, h->hbn, 1, h->st);
-    }));
-    bool widen = true;
-    TRY(sap_half_widen(h, k, 1, &widen));
+    bool blocks = true;
+    TRY(sap32_by_blocks(h, (const float*)h->fin, (float*)h->fout, 1, &blocks));
   }
   return DDAMG_OK;
 }
@@ -2840,41 +2808,24 @@ ddamg_status ddamg_block_solve(ddamg_handle h, int prec, int colour, int nrhs, c
                                int on_device) {
   if (!h || nrhs < 1 || !in || !out || (colour != 0 && colour != 1)) return DDAMG_EINVAL;
   const int k = half_kind(prec);
-  if (k >= 0 && sap_half_ok(h->g)) {
-    TRY(need_tmp(h, nrhs, 6));
-    TRY(half_operators(h, k));
-    TRY(need_half_fields(h, nrhs));
-    float* t0 = (float*)h->tmp[0];
-    TRY(import_fields<float>(h, in, on_device, nrhs, t0));
-    CK(by_half(k, [&](auto* tag) {
-      using S = std::remove_pointer_t<decltype(tag)>;
-      return spinor_to_half<S>(h->g, t0, h->hb, h->hbn, nrhs, h->st);
-    }));
-    bool widen = true;
-    TRY(sap_half_widen(h, k, nrhs, &widen));
-    CK(cudaMemsetAsync(h->hx, 0, nrhs * h->V24 * 2, h->st));
-    CK(cudaMemsetAsync(h->hxn, 0, nrhs * h->g.V * sizeof(float), h->st));
-    ++h->n_cls[1];
-    CK(by_half(k, [&](auto* tag) {
-      using S = std::remove_pointer_t<decltype(tag)>;
-      cudaError_t e = sap_sweep_h<S>(h->g, colour, h->p.mr_iters, true, h->hb, h->hbn, h->hx, h->hxn, h->gH[k],
-                                     h->AH[k], h->AiH[k], nrhs, h->d_status, h->wait_sap, h->st, widen);
-      if (e != cudaSuccess) return e;
-      return spinor_from_half<S>(h->g, h->hx, h->hxn, t0, nrhs, false, h->st);
-    }));
-    TRY(check_status(h));
-    return export_fields<float>(h, t0, nrhs, out, on_device);
-  }
   return dispatch(h, prec, [&](auto* tag) -> ddamg_status {
     using R = std::remove_pointer_t<decltype(tag)>;
     TRY(need_tmp(h, nrhs, 6));
+    if (k >= 0 && sap_block_ok(h->g)) TRY(half_operators(h, k));
     R* b = (R*)h->tmp[0];
     R* x = (R*)h->tmp[1];
     TRY(import_fields<R>(h, in, on_device, nrhs, b));
     CK(cudaMemsetAsync(x, 0, nrhs * h->V24 * sizeof(R), h->st));
     ++h->n_cls[1];
-    CK(sap_sweep<R>(h->g, colour, h->p.mr_iters, true, b, x, gauge_of<R>(h), clov_of<R>(h, false),
-                    clov_of<R>(h, true), nrhs, h->d_status, h->wait_sap, h->st));
+    if (sizeof(R) == 4 && sap_block_ok(h->g)) {
+      const SapStep s{1, 0, 0, 0, true};
+      CK(sap_block_sweep(h->g, k, colour, h->p.mr_iters, s, (const float*)b, (float*)x, nullptr, nullptr,
+                         k >= 0 ? h->gH[k] : h->g32, k >= 0 ? h->AH[k] : h->A32, k >= 0 ? h->AiH[k] : h->Ai32, nrhs,
+                         h->d_status, h->wait_sap, h->st));
+    } else {
+      CK(sap_sweep<R>(h->g, colour, h->p.mr_iters, true, b, x, gauge_of<R>(h), clov_of<R>(h, false),
+                      clov_of<R>(h, true), nrhs, h->st));
+    }
     TRY(check_status(h));
     return export_fields<R>(h, x, nrhs, out, on_device);
   });

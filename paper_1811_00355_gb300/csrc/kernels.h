@@ -171,27 +171,35 @@ cudaError_t index_maps(const Geom& g, int* parity, int* block, int* colour, cuda
 // one colour of a Schwarz sweep on all blocks of that colour:
 //   r = b - D x (or r = b if x_is_zero), e = MR-even-odd block solve of r,
 //   x += e (x is overwritten with e if x_is_zero)
-// *status receives DDAMG_ETIMEOUT (6) if a bounded wait for staged data gives
-// up after wait_limit polls (the CTA then leaves x untouched)
-// (staged: the FP32 kernel with the block's links and clover blocks staged
-// in shared memory where the block shape allows it, else the general one)
+// (any block shape, FP64 and FP32)
 template <class R>
 cudaError_t sap_sweep(const Geom& g, int colour, int mr_iters, bool x_is_zero, const R* b,
-                      R* x, const R* gauge, const R* clover, const R* clover_inv, int nrhs,
-                      int* status, long long wait_limit, cudaStream_t st, bool staged = true);
-// the staged FP32 kernel applies to the block shape of g
-bool sap_staged_ok(const Geom& g);
+                      R* x, const R* gauge, const R* clover, const R* clover_inv, int nrhs, cudaStream_t st);
 size_t sap_smem_bytes(const Geom& g, int real_size);
-// one colour of a Schwarz sweep with half storage (FP32 arithmetic): links,
-// clover blocks A and A^-1 and the spinors b, x (with their site norms) in
-// the half type S; needs blocks whose half volume is a multiple of 32.
-// widen: the staged block operators are widened to FP32 in shared memory
-// (where the FP32 staging fits the block), else kept in the half type
-template <class S>
-cudaError_t sap_sweep_h(const Geom& g, int colour, int mr_iters, bool x_is_zero, const void* b, const float* bn,
-                        void* x, float* xn, const void* gauge, const void* clover, const void* clover_inv, int nrhs,
-                        int* status, long long wait_limit, cudaStream_t st, bool widen = true);
-bool sap_half_ok(const Geom& g);
+// The same sweep in FP32 for blocks of 64, 128, 192 or 256 sites, with the
+// residual carried from sweep to sweep instead of recomputed: between its
+// sweeps a block keeps its even residual (res; the odd one is zero after a
+// block solve), and the blocks of the other colour leave what their update
+// sends across their faces (msg).  Links and clover blocks in FP32
+// (half_kind -1), FP16 (0) or BF16 (1); FP32 fields.
+struct SapStep {
+  int first;      // the colour's first sweep: r starts from b and x is overwritten
+  int take;       // the other colour has updated x since: add its messages
+  int give;       // the other colour sweeps again: leave messages
+  int keep;       // this colour sweeps again: leave the even residual
+  bool overlap;   // the kernel before may still run while the operators are loaded
+                  // (it must not be the one that wrote them)
+};
+// *status receives DDAMG_ETIMEOUT (6) if a bounded wait for staged data gives
+// up after wait_limit polls (the CTA then leaves its outputs untouched)
+cudaError_t sap_block_sweep(const Geom& g, int half_kind, int colour, int mr_iters, const SapStep& step, const float* b,
+                            float* x, void* res, void* msg, const void* gauge, const void* clover,
+                            const void* clover_inv, int nrhs, int* status, long long wait_limit, cudaStream_t st);
+// the block shape of g has this form
+bool sap_block_ok(const Geom& g);
+// bytes per right-hand side of res and msg: at most 192 a site
+size_t sap_res_bytes(const Geom& g);
+size_t sap_msg_bytes(const Geom& g);
 
 // ---- third level (kernels_level2.cu) ----------------------------------------------
 // The coarse lattice of level 1 cut into blocks of coarse sites (the level-2

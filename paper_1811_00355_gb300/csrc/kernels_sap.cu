@@ -2,8 +2,9 @@
 // multiplicative Schwarz sweep over the blocks of one colour, the block
 // system solved approximately by site even-odd preconditioned minimal
 // residual with a fixed number of iterations.  Loops over blocks are the
-// parallel dimension (Sec. 4); here one CTA owns one block and one
-// right-hand side, with the block's links staged in shared memory.
+// parallel dimension (Sec. 4); here one CTA owns one block.  Two kernels: the
+// general one (any block shape, FP64 and FP32, one right-hand side per CTA,
+// the block's links in shared memory), and the FP32 block kernel further down.
 //
 // Per CTA (block B of colour c):
 //   r   = b - D x on the block's sites (full operator, neighbours from global
@@ -481,53 +482,540 @@ __global__ void __launch_bounds__(512) k_sap_sweep(Geom g, int colour, int mr_it
 }
 
 // ---------------------------------------------------------------------------
-// Staged sweep (FP32 arithmetic) for Schwarz blocks whose half volume is a
-// multiple of 32: the thread layout and hop code of k_sap_sweep (four
-// threads per site, one runtime direction each, partial sums combined by
-// warp shuffles), with
-//  * the block's links, A_ee and A_oo^-1 staged into shared memory by bulk
-//    asynchronous copies (cp.async.bulk + mbarrier) that land while the
-//    residual is computed from global memory;
-//  * each thread's block-internal neighbour indices held in registers;
-//  * a programmatic-dependent-launch prologue: barrier set-up and the staging
-//    copies (links and clover are read-only during a solve) are issued before
-//    griddepcontrol.wait, so they overlap the previous sweep's tail.
-// Storage S: FP32 (16-byte units), or BF16 / FP16 (half.cuh: 8-byte units of
-// the same four values, spinors divided by their site norms).
+// Block kernel (FP32 arithmetic) for Schwarz blocks of 64, 128, 192 or 256
+// sites: a thread per site, the site's links and its clover block (A_ee on an
+// even site, A_oo^-1 on an odd one) in registers for the whole launch.
+//
+// What bounds it: instruction issue and latency of few warps.  The block
+// solve has about 3 MFLOP but 36 half-spinor exchanges with barriers between
+// them; a block's operators (120 KB) come from L2 or DRAM once per launch.
+// The form before (four threads per site, operators read from shared memory
+// at every hop, the residual b - D x recomputed from global memory in every
+// sweep) spent 640 instructions per thread and hop phase on selects, shuffles
+// and shared-memory reads: 34 us per sweep of one right-hand side on 16^4,
+// 35 us per block solve on 24^3 x 48.  This one: 21 us and 17.6 us.
+//  * A thread multiplies only with its own four links: forward hops as the
+//    receiver, backward ones as the sender, so a link is held once and both
+//    parities work at the same time (half steps below).
+//  * Hops leaving the block read a place of zeros instead of branching.
+//  * The residual is carried: after a block solve it is zero on the odd sites
+//    and the MR residual on the even ones, and only hops across block faces
+//    change it until the block's next sweep.  Every sweep leaves those hops as
+//    half spinors (msg) for the other colour, a quarter of the hops of a 4^4
+//    block and no clover product.  (Error of the smoother against 64 bits on
+//    the lattices above 1.8e-7, with recomputed residuals 1.5e-7.)
+//  * What the next right-hand side needs arrives by bulk copies while this one
+//    is solved.
+//  * The loop's parts exist once each, or the code would not stay in the
+//    instruction cache: with every use inlined the same algorithm took 26 us.
+// Two threads per site (two links and one chirality each, 512 threads) were
+// slower, 24 us: twice the shared-memory traffic, and registers spilled.
 // ---------------------------------------------------------------------------
+namespace blk {
+
+using f2 = cpx<float>;
+
+struct SapArgs {
+  Geom g;
+  int colour, mr_iters, nrhs, per;   // right-hand sides of the call and per CTA
+  int first, take, give, keep;
+  const float* b;
+  float* x;
+  float4* res;
+  float4* msg;
+  const void* gauge;
+  const void* clov;
+  const void* clov_inv;
+  int* status;
+  long long wait_limit;
+};
+
+// staged operator units of site q (half h) -> links (halved) and clover block
+template <class S>
+struct Ops;
+template <>
+struct Ops<float> {
+  using T = float4;
+  static constexpr int LU = 12, CU = 18;
+  __device__ __forceinline__ static void links(const T* sl, int Vb, int q, Link<float> (&U)[4]) {
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+      const float4 a = sl[(3 * m) * Vb + q], b = sl[(3 * m + 1) * Vb + q], c = sl[(3 * m + 2) * Vb + q];
+      U[m].m[0][0] = mk(a.x, a.y); U[m].m[0][1] = mk(a.z, a.w); U[m].m[0][2] = mk(b.x, b.y);
+      U[m].m[1][0] = mk(b.z, b.w); U[m].m[1][1] = mk(c.x, c.y); U[m].m[1][2] = mk(c.z, c.w);
+    }
+  }
+  __device__ __forceinline__ static void clover(const T* A, int Vh, int h, float (&P)[72]) {
+#pragma unroll
+    for (int u = 0; u < 18; ++u) {
+      const float4 a = A[u * Vh + h];
+      P[4 * u] = a.x; P[4 * u + 1] = a.y; P[4 * u + 2] = a.z; P[4 * u + 3] = a.w;
+    }
+  }
+};
+template <class S>
+struct OpsHalf {
+  using T = uint4;
+  static constexpr int LU = HGAUGE_NU, CU = HCLOV_NU;
+  __device__ __forceinline__ static void links(const T* sl, int Vb, int q, Link<float> (&U)[4]) {
+    float v[48];
+#pragma unroll
+    for (int u = 0; u < 6; ++u) unpack8<S>(sl[u * Vb + q], v + 8 * u);
+#pragma unroll
+    for (int m = 0; m < 4; ++m)
+#pragma unroll
+      for (int k = 0; k < 6; ++k) U[m].m[k / 3][k % 3] = mk(v[12 * m + 2 * k], v[12 * m + 2 * k + 1]);
+  }
+  __device__ __forceinline__ static void clover(const T* A, int Vh, int h, float (&P)[72]) {
+#pragma unroll
+    for (int u = 0; u < 9; ++u) unpack8<S>(A[u * Vh + h], P + 8 * u);
+  }
+};
+template <>
+struct Ops<__half> : OpsHalf<__half> {};
+template <>
+struct Ops<__nv_bfloat16> : OpsHalf<__nv_bfloat16> {};
+
+__device__ __forceinline__ void put_half(float4* p, int stride, const f2 (&h)[2][3]) {
+  p[0] = make_float4(h[0][0].re, h[0][0].im, h[0][1].re, h[0][1].im);
+  p[stride] = make_float4(h[0][2].re, h[0][2].im, h[1][0].re, h[1][0].im);
+  p[2 * stride] = make_float4(h[1][1].re, h[1][1].im, h[1][2].re, h[1][2].im);
+}
+__device__ __forceinline__ void as_half(const float4& a, const float4& b, const float4& c, f2 (&h)[2][3]) {
+  h[0][0] = mk(a.x, a.y); h[0][1] = mk(a.z, a.w); h[0][2] = mk(b.x, b.y);
+  h[1][0] = mk(b.z, b.w); h[1][1] = mk(c.x, c.y); h[1][2] = mk(c.z, c.w);
+}
+__device__ __forceinline__ void get_half(const float4* p, int stride, f2 (&h)[2][3]) {
+  as_half(p[0], p[stride], p[2 * stride], h);
+}
+
+// U^H (1 + g_MU) psi for the site ahead, one direction after the other
+template <int MU>
+__device__ __forceinline__ void ahead_dir(const Spinor<float>& psi, const Link<float>& U, float4* gx, int row, int h) {
+  f2 hh[2][3], y[2][3];
+  project<MU, +1>(psi, hh);
+  su3_mul_dag(U, hh, y);
+  put_half(gx + (size_t)(3 * MU) * row + h, row, y);
+}
+__device__ __forceinline__ void send_ahead(const Spinor<float>& psi, const Link<float> (&U)[4], float4* gx, int row, int h) {
+  ahead_dir<0>(psi, U[0], gx, row, h);
+  ahead_dir<1>(psi, U[1], gx, row, h);
+  ahead_dir<2>(psi, U[2], gx, row, h);
+  ahead_dir<3>(psi, U[3], gx, row, h);
+}
+// acc += (1 - g_MU) U psi(ahead) from the published spinors (n: the
+// neighbours' places); a direction's spinor is loaded while the one before is
+// multiplied
+__device__ __forceinline__ void load6(const float4* p, int stride, Spinor<float>& s) {
+#pragma unroll
+  for (int u = 0; u < 6; ++u) {
+    const float4 a = p[u * stride];
+    s.c[2 * u] = mk(a.x, a.y);
+    s.c[2 * u + 1] = mk(a.z, a.w);
+  }
+}
+template <int MU>
+__device__ __forceinline__ void fwd_dir(Spinor<float>& acc, const Link<float>& U, const Spinor<float>& nb) {
+  f2 hh[2][3], y[2][3];
+  project<MU, -1>(nb, hh);
+  su3_mul(U, hh, y);
+  accumulate<MU, -1>(acc, y, 1.f);
+}
+__device__ __forceinline__ void take_ahead(Spinor<float>& acc, const Link<float> (&U)[4], const float4* pub, int row,
+                                           unsigned n0, unsigned n1) {
+  Spinor<float> p, q;
+  load6(pub + (n0 & 255u), row, p);
+  load6(pub + ((n0 >> 16) & 255u), row, q);
+  fwd_dir<0>(acc, U[0], p);
+  load6(pub + (n1 & 255u), row, p);
+  fwd_dir<1>(acc, U[1], q);
+  load6(pub + ((n1 >> 16) & 255u), row, q);
+  fwd_dir<2>(acc, U[2], p);
+  fwd_dir<3>(acc, U[3], q);
+}
+// acc += the half spinors that the sites behind sent ahead
+template <int MU>
+__device__ __forceinline__ void bwd_dir(Spinor<float>& acc, const float4* gx, int row, unsigned n) {
+  f2 hh[2][3];
+  get_half(gx + (size_t)(3 * MU) * row + n, row, hh);
+  accumulate<MU, +1>(acc, hh, 1.f);
+}
+__device__ __forceinline__ void take_behind(Spinor<float>& acc, const float4* gx, int row, unsigned n0, unsigned n1) {
+  bwd_dir<0>(acc, gx, row, (n0 >> 8) & 255u);
+  bwd_dir<1>(acc, gx, row, n0 >> 24);
+  bwd_dir<2>(acc, gx, row, (n1 >> 8) & 255u);
+  bwd_dir<3>(acc, gx, row, n1 >> 24);
+}
+
+__device__ __forceinline__ void clover12(const float (&P)[72], const Spinor<float>& v, Spinor<float>& y) {
+  herm6<float>(P, v.c, y.c);
+  herm6<float>(P + 36, v.c + 6, y.c + 6);
+}
+
+__device__ __forceinline__ void bar_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
+
+__device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+
+// the hops of direction MU from the neighbouring blocks: their messages, the
+// lower face of the block ahead and the upper face of the block behind (sites
+// inside the block take zeros)
+template <int MU>
+__device__ __forceinline__ void outer_dir(Spinor<float>& r, const Link<float>& U, const float4* m, const float4* zero,
+                                          bool lower, bool upper, int F, float sf, float sb) {
+  f2 hh[2][3], y[2][3], bb[2][3];
+  const float4 *pf = upper ? m : zero, *pb = lower ? m + 3 * F : zero;
+  get_half(pf, upper ? F : 0, hh);
+  get_half(pb, lower ? F : 0, bb);
+  su3_mul(U, hh, y);
+  accumulate<MU, -1>(r, y, MU == 3 ? sf : 1.f);
+  accumulate<MU, +1>(r, bb, MU == 3 ? sb : 1.f);
+}
+// and what this site sends them
+template <int MU>
+__device__ __forceinline__ void give_dir(const Spinor<float>& v, const Link<float>& U, float4* m, bool lower, bool upper,
+                                         int F) {
+  f2 hh[2][3], y[2][3];
+  if (lower) {
+    project<MU, -1>(v, hh);
+    put_half(m, F, hh);
+  }
+  if (upper) {
+    project<MU, +1>(v, hh);
+    su3_mul_dag(U, hh, y);
+    put_half(m + 3 * F, F, y);
+  }
+}
+
+// float4 units of a block's messages: three per site of each face
+__host__ __device__ __forceinline__ int msg_units(const Geom& g) {
+  return 6 * (g.Vb / g.b[0] + g.Vb / g.b[1] + g.Vb / g.b[2] + g.Vb / g.b[3]);
+}
+
+// VB: the block's sites if known at compile time (4^4 blocks: constant strides
+// take 10 % off the solve), else 0
+template <class S, int VB>
+__global__ void __launch_bounds__(256, 1) k_sap_block(SapArgs a) {
+  using T = typename Ops<S>::T;
+  constexpr int LU = Ops<S>::LU, CU = Ops<S>::CU;
+  constexpr unsigned UB = sizeof(T);
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const Geom& g = a.g;
+  const int Vb = VB ? VB : g.Vb, Vh = Vb / 2, row = Vh + 1, S3 = msg_units(g);
+  float4* pub = reinterpret_cast<float4*>(smem_raw);       // [parity][6][Vh + 1] published spinors
+  float4* gx = pub + 12 * row;                             // [parity][12][Vh + 1] sent ahead
+  float4* red = gx + 24 * row;                             // [warps of one parity]
+  float4* area = red + Vh / 32;                            // staged operators, then:
+  float4* kp = area;                                       // [6][Vb] kept -r_o / e_e
+  float4* base = kp + 6 * Vb;                              // [6][Vb] b, or [6][Vh] the even residual
+  float4* xs = base + 6 * Vb;                              // [6][Vb] x
+  float4* ms = xs + 6 * Vb;                                // [S3] the neighbours' messages
+  T* sl = reinterpret_cast<T*>(area);                      // [LU][Vb]
+  T* Aee = sl + LU * Vb;                                   // [CU][Vh]
+  T* Aoi = Aee + CU * Vh;                                  // [CU][Vh]
+
+  const int t = threadIdx.x;
+  const bool odd = t >= Vh;
+  const int h = odd ? t - Vh : t;
+  const int slices = gridDim.x / (g.nb / 2);
+  const int B = block_of_colour(g, a.colour, blockIdx.x / slices);
+  const int rhs0 = (blockIdx.x % slices) * a.per, rhs1 = min(a.nrhs, rhs0 + a.per);
+
+  __shared__ __align__(8) uint64_t bar_ops, bar_in, bar_x;
+  __shared__ float2 alpha;                                 // the last MR step's
+  if (t < 32) {
+    if (t == 0) {
+      mbar_init(&bar_ops, 1);
+      mbar_init(&bar_in, 1);
+      mbar_init(&bar_x, 1);
+      mbar_fence_init();
+    }
+    __syncwarp();
+    const unsigned links = (unsigned)(LU * Vb) * UB, half = (unsigned)Vh * UB;
+    if (t == 0) {
+      mbar_expect_tx(&bar_ops, links + 2u * CU * half);
+      bulk_g2s(sl, reinterpret_cast<const T*>(a.gauge) + (size_t)B * LU * Vb, links, &bar_ops);
+    }
+    const T* ca = reinterpret_cast<const T*>(a.clov) + (size_t)B * CU * Vb;
+    const T* ci = reinterpret_cast<const T*>(a.clov_inv) + (size_t)B * CU * Vb + Vh;
+    for (int u = t; u < 2 * CU; u += 32) {
+      if (u < CU) bulk_g2s(Aee + u * Vh, ca + (size_t)u * Vb, half, &bar_ops);
+      else bulk_g2s(Aoi + (u - CU) * Vh, ci + (size_t)(u - CU) * Vb, half, &bar_ops);
+    }
+  }
+  // the place past the last one stands for a neighbour outside the block
+  if (t < 36) pub[t * row + Vh] = make_float4(0.f, 0.f, 0.f, 0.f);
+  launch_dependents();
+  // places of the eight block-internal neighbours among the other parity's sites
+  unsigned n0 = 0, n1 = 0;
+#pragma unroll
+  for (int m = 0; m < 4; ++m) {
+    int f = __ldg(g.bnbr + (2 * m) * Vb + t), b = __ldg(g.bnbr + (2 * m + 1) * Vb + t);
+    f = f < 0 ? Vh : (f >= Vh ? f - Vh : f);
+    b = b < 0 ? Vh : (b >= Vh ? b - Vh : b);
+    const unsigned w = (unsigned)f | ((unsigned)b << 8);
+    if (m < 2) n0 |= w << (16 * m);
+    else n1 |= w << (16 * (m - 2));
+  }
+  auto outside = [&](unsigned n, int sh) { return ((n >> sh) & 255u) == (unsigned)Vh; };
+  // this site's place among the messages of a face, by direction
+  int pos[4];
+  const int F0 = Vb / g.b[0], F1 = Vb / g.b[1], F2 = Vb / g.b[2], F3 = Vb / g.b[3];
+  {
+    int l[4], r = h;
+    l[0] = 2 * (r % (g.b[0] / 2)); r /= g.b[0] / 2;
+    l[1] = r % g.b[1]; r /= g.b[1];
+    l[2] = r % g.b[2]; l[3] = r / g.b[2];
+    l[0] += ((odd ? 1 : 0) + l[1] + l[2] + l[3]) & 1;
+    pos[0] = l[1] + g.b[1] * (l[2] + g.b[2] * l[3]);
+    pos[1] = 6 * F0 + l[0] + g.b[0] * (l[2] + g.b[2] * l[3]);
+    pos[2] = 6 * (F0 + F1) + l[0] + g.b[0] * (l[1] + g.b[1] * l[3]);
+    pos[3] = 6 * (F0 + F1 + F2) + l[0] + g.b[0] * (l[1] + g.b[1] * l[2]);
+  }
+  // b or the even residual (lane 8) and the messages (lanes 0 .. 7, a face each)
+  const int face = t & 7, fF = Vb / g.b[face >> 1];
+  int foff = 3 * fF * (face & 1);
+  for (int m = 0; m < (face >> 1); ++m) foff += 6 * (Vb / g.b[m]);
+  const int fY = __ldg(g.cnbr + (1 + face) * g.nb + B);
+  // sign of the hops across the time boundary (t runs slowest over the blocks)
+  const float sf = __ldg(g.cnbr + 7 * g.nb + B) < B ? -1.f : 1.f, sb = __ldg(g.cnbr + 8 * g.nb + B) > B ? -1.f : 1.f;
+  __syncthreads();
+  // false when a copy did not land in time: the status is set and every copy
+  // in flight has been waited for
+  auto landed = [&](uint64_t* bar, unsigned phase, int in_phase, int x_phase) -> bool {
+    const bool ok = mbar_wait_bounded(bar, phase, a.wait_limit);
+    if (!__syncthreads_or(!ok)) return true;
+    if (t == 0) atomicExch(a.status, 6);
+    mbar_wait_bounded(&bar_ops, 0, MBAR_POLL_LIMIT);
+    if (in_phase >= 0) mbar_wait_bounded(&bar_in, in_phase & 1, MBAR_POLL_LIMIT);
+    if (x_phase >= 0) mbar_wait_bounded(&bar_x, x_phase & 1, MBAR_POLL_LIMIT);
+    return false;
+  };
+  if (!landed(&bar_ops, 0, -1, -1)) return;
+  Link<float> U[4];
+  float P[72];
+  Ops<S>::links(sl, Vb, t, U);
+  Ops<S>::clover(odd ? Aoi : Aee, Vh, h, P);
+  if (odd)
+#pragma unroll
+    for (int k = 0; k < 72; ++k) P[k] = -P[k];
+#pragma unroll
+  for (int m = 0; m < 4; ++m) {
+    complete_link(U[m]);
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+      for (int j = 0; j < 3; ++j) U[m].m[i][j] = 0.5f * U[m].m[i][j];
+  }
+  __syncthreads();       // the staged operators are in registers: their place is free
+  grid_dependency_wait();
+
+  auto fetch_in = [&](int rhs) {
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    if (t == 8) {
+      const size_t blk = (size_t)rhs * g.nb + B;
+      const unsigned nb = (unsigned)(a.first ? 6 * Vb : 6 * Vh) * 16u;
+      mbar_expect_tx(&bar_in, nb + (a.take ? (unsigned)S3 * 16u : 0u));
+      bulk_g2s(base, a.first ? reinterpret_cast<const float4*>(a.b) + blk * 6 * Vb : a.res + blk * 6 * Vh, nb, &bar_in);
+    } else if (a.take) {
+      bulk_g2s(ms + foff, a.msg + ((size_t)rhs * g.nb + fY) * S3 + foff, 3u * fF * 16u, &bar_in);
+    }
+  };
+  if (t < 9) fetch_in(rhs0);
+  for (int rhs = rhs0; rhs < rhs1; ++rhs) {
+    const size_t blk = (size_t)rhs * g.nb + B;
+    float4* xb = reinterpret_cast<float4*>(a.x) + blk * 6 * Vb;
+    if (t == 0 && !a.first) {
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      mbar_expect_tx(&bar_x, 6u * Vb * 16u);
+      bulk_g2s(xs, xb, 6u * Vb * 16u, &bar_x);
+    }
+    const int n = rhs - rhs0;
+    if (!landed(&bar_in, n & 1, n, a.first ? -1 : n)) return;
+    Spinor<float> v, out;
+    if (a.first || !odd) {
+      const float4* p = a.first ? base + t : base + h;
+      const int st = a.first ? Vb : Vh;
+#pragma unroll
+      for (int u = 0; u < 6; ++u) {
+        const float4 q = p[u * st];
+        out.c[2 * u] = mk(q.x, q.y);
+        out.c[2 * u + 1] = mk(q.z, q.w);
+      }
+    } else {
+#pragma unroll
+      for (int k = 0; k < 12; ++k) out.c[k] = mk(0.f, 0.f);
+    }
+    if (a.take) {
+      outer_dir<0>(out, U[0], ms + pos[0], pub + Vh, outside(n0, 8), outside(n0, 0), F0, sf, sb);
+      outer_dir<1>(out, U[1], ms + pos[1], pub + Vh, outside(n0, 24), outside(n0, 16), F1, sf, sb);
+      outer_dir<2>(out, U[2], ms + pos[2], pub + Vh, outside(n1, 8), outside(n1, 0), F2, sf, sb);
+      outer_dir<3>(out, U[3], ms + pos[3], pub + Vh, outside(n1, 24), outside(n1, 16), F3, sf, sb);
+    }
+    if (odd)
+#pragma unroll
+      for (int k = 0; k < 12; ++k) out.c[k] = -out.c[k];
+#pragma unroll
+    for (int u = 0; u < 6; ++u)
+      kp[u * Vb + t] = odd ? make_float4(out.c[2 * u].re, out.c[2 * u].im, out.c[2 * u + 1].re, out.c[2 * u + 1].im)
+                           : make_float4(0.f, 0.f, 0.f, 0.f);
+    v = out;
+    // The even-odd solve in half steps: at an even one the even sites receive
+    // a hop from the odd ones, at an odd one the odd sites from the even ones.
+    // While the receivers multiply their own links with the spinors ahead,
+    // the senders multiply theirs for the sites ahead of them, so all warps
+    // work; then the receivers add what was sent and make the next vector.
+    //   odd   -1: w = A_oo^-1 r_o      2 i - 1: q_i = 1/2 hop res, w = -A_oo^-1 q_i
+    //   even  0: res = r_e + 1/2 hop w      2 i: p = A_ee res + 1/2 hop w, MR step alpha_i
+    //   odd   2 m + 1: e_o = A_oo^-1 (r_o + sum alpha_i q_i), the hop of e_e
+    //         being the sum of the alpha_i times those of the residuals
+    // with -A_oo^-1 as the odd block and -r_o in its place, so that every hop
+    // is added.  One copy of each part's code serves both parities: the loop
+    // has to stay in the instruction cache.
+    const int m = a.mr_iters;
+    float4* my_pub = odd ? pub + 6 * row : pub;
+    float4* my_gx = odd ? gx + 12 * row : gx;
+    const float4* th_pub = odd ? pub : pub + 6 * row;
+    const float4* th_gx = odd ? gx : gx + 12 * row;
+    // odd: q_i (in out) joins the kept vector once alpha_i is known
+    auto keep_q = [&]() {
+      const f2 al = mk(alpha.x, alpha.y);
+#pragma unroll
+      for (int u = 0; u < 6; ++u) {
+        const float4 z = kp[u * Vb + t];
+        f2 x0 = mk(z.x, z.y), x1 = mk(z.z, z.w);
+        x0 = x0 - al * out.c[2 * u];
+        x1 = x1 - al * out.c[2 * u + 1];
+        kp[u * Vb + t] = make_float4(x0.re, x0.im, x1.re, x1.im);
+      }
+    };
+    for (int hs = -1;; ++hs) {
+      const bool rx = ((hs & 1) != 0) == odd;
+      if (hs > 1 && odd && rx) keep_q();
+      if (hs >= 0 && hs <= 2 * m) {
+        if (!rx) {
+          send_ahead(v, U, my_gx, row, h);
+        } else {
+          if (odd)
+#pragma unroll
+            for (int k = 0; k < 12; ++k) out.c[k] = mk(0.f, 0.f);
+          take_ahead(out, U, th_pub, row, n0, n1);
+        }
+        __syncthreads();
+        if (rx) take_behind(out, th_gx, row, n0, n1);
+      }
+      if (hs == 2 * m + 1 && odd) {
+#pragma unroll
+        for (int u = 0; u < 6; ++u) {
+          const float4 q = kp[u * Vb + t];
+          out.c[2 * u] = mk(q.x, q.y);
+          out.c[2 * u + 1] = mk(q.z, q.w);
+        }
+      }
+      if (hs & 1) {
+        // both parities multiply their own block: w or e_o, and A_ee res
+        if (odd) clover12(P, out, v);
+        else if (hs > 0 && hs < 2 * m + 1) clover12(P, v, out);
+      } else if (!odd) {
+        if (hs == 0) {
+          v = out;
+        } else {
+          load6(my_pub + h, row, v);        // res
+          float d[6] = {};
+#pragma unroll
+          for (int k = 0; k < 12; ++k) {
+            const int e = 3 * (k & 1);
+            d[e] = fmaf(out.c[k].re, v.c[k].re, fmaf(out.c[k].im, v.c[k].im, d[e]));
+            d[e + 1] = fmaf(out.c[k].re, v.c[k].im, fmaf(-out.c[k].im, v.c[k].re, d[e + 1]));
+            d[e + 2] = fmaf(out.c[k].re, out.c[k].re, fmaf(out.c[k].im, out.c[k].im, d[e + 2]));
+          }
+          float sre = d[0] + d[3], sim = d[1] + d[4], spp = d[2] + d[5];
+          sre = warp_sum_r<float>(sre);
+          sim = warp_sum_r<float>(sim);
+          spp = warp_sum_r<float>(spp);
+          if ((t & 31) == 0) red[t >> 5] = make_float4(sre, sim, spp, 0.f);
+          bar_sync(1, Vh);
+          sre = sim = spp = 0.f;
+          for (int w = 0; w < Vh / 32; ++w) {
+            const float4 q = red[w];
+            sre += q.x; sim += q.y; spp += q.z;
+          }
+          if (spp > 0.f) {
+            const float inv = 1.f / spp;
+            const f2 al = mk(sre * inv, sim * inv);
+            if (t == 0) alpha = make_float2(al.re, al.im);
+#pragma unroll
+            for (int u = 0; u < 6; ++u) {
+              const float4 q = kp[u * Vb + t];
+              f2 x0 = mk(q.x, q.y), x1 = mk(q.z, q.w);
+              fma(x0, al, v.c[2 * u]);
+              fma(x1, al, v.c[2 * u + 1]);
+              kp[u * Vb + t] = make_float4(x0.re, x0.im, x1.re, x1.im);
+            }
+#pragma unroll
+            for (int k = 0; k < 12; ++k) v.c[k] = v.c[k] - al * out.c[k];
+          } else if (t == 0) {
+            alpha = make_float2(0.f, 0.f);
+          }
+        }
+        if (hs == 2 * m) {
+          if (a.keep) {
+            float4* rb = a.res + blk * 6 * Vh + h;
+#pragma unroll
+            for (int u = 0; u < 6; ++u)
+              rb[u * Vh] = make_float4(v.c[2 * u].re, v.c[2 * u].im, v.c[2 * u + 1].re, v.c[2 * u + 1].im);
+          }
+#pragma unroll
+          for (int u = 0; u < 6; ++u) {
+            const float4 q = kp[u * Vb + t];
+            v.c[2 * u] = mk(q.x, q.y);
+            v.c[2 * u + 1] = mk(q.z, q.w);
+          }
+        }
+      }
+      if (hs == 2 * m + 1) break;
+      if (rx && hs < 2 * m)
+#pragma unroll
+        for (int u = 0; u < 6; ++u)
+          my_pub[u * row + h] = make_float4(v.c[2 * u].re, v.c[2 * u].im, v.c[2 * u + 1].re, v.c[2 * u + 1].im);
+      __syncthreads();
+      if (hs < 0 && t < 9 && rhs + 1 < rhs1) fetch_in(rhs + 1);     // everyone has read this one's
+    }
+    // v = e_o or e_e
+    if (a.give) {
+      float4* to = a.msg + blk * S3;
+      give_dir<0>(v, U[0], to + pos[0], outside(n0, 8), outside(n0, 0), F0);
+      give_dir<1>(v, U[1], to + pos[1], outside(n0, 24), outside(n0, 16), F1);
+      give_dir<2>(v, U[2], to + pos[2], outside(n1, 8), outside(n1, 0), F2);
+      give_dir<3>(v, U[3], to + pos[3], outside(n1, 24), outside(n1, 16), F3);
+    }
+    if (!a.first && !landed(&bar_x, n & 1, n + 1 < rhs1 - rhs0 ? n + 1 : n, n)) return;
+#pragma unroll
+    for (int u = 0; u < 6; ++u) {
+      float4 q = a.first ? make_float4(0.f, 0.f, 0.f, 0.f) : xs[u * Vb + t];
+      q.x += v.c[2 * u].re;
+      q.y += v.c[2 * u].im;
+      q.z += v.c[2 * u + 1].re;
+      q.w += v.c[2 * u + 1].im;
+      xb[u * Vb + t] = q;
+    }
+    if (rhs + 1 < rhs1) __syncthreads();       // x and the sent half spinors have been read
+  }
+}
+
+}  // namespace blk
+
 namespace stg {
 
 using f2 = cpx<float>;
 
-// storage traits: unit type of the staged arrays and global loads / stores
+// loads and stores by storage type: FP32, or BF16 / FP16 (half.cuh; spinors
+// divided by their site norms)
 template <class S>
 struct IO;
 template <>
 struct IO<float> {
-  using T = float4;
-  static constexpr int LINK_U = 12;   // 16-byte units per site: links
-  static constexpr int CLOV_U = 18;   // clover blocks
-  __device__ __forceinline__ static void unpack(const T& t, float* v) {
-    v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
-  }
-  // 36 values of chiral block cb from a staged clover array ([units][Vh], site h)
-  __device__ __forceinline__ static void block_smem(const T* A, int Vh, int h, int cb, float* P) {
-#pragma unroll
-    for (int u = 0; u < 9; ++u) unpack(A[(9 * cb + u) * Vh + h], P + 4 * u);
-  }
-  // rows 0 and 1 of link mu of local site q from the staged links (rows of
-  // Vbp units); link_smem also rebuilds row 2
-  __device__ __forceinline__ static void link2_smem(const T* sl, int Vbp, int q, int mu, Link<float>& U) {
-    float v[LINK_NR];
-#pragma unroll
-    for (int u = 0; u < 3; ++u) unpack(sl[(mu * 3 + u) * Vbp + q], v + 4 * u);
-#pragma unroll
-    for (int k = 0; k < 6; ++k) U.m[k / 3][k % 3] = mk(v[2 * k], v[2 * k + 1]);
-  }
-  __device__ __forceinline__ static void link_smem(const T* sl, int Vbp, int q, int mu, Link<float>& U) {
-    link2_smem(sl, Vbp, q, mu, U);
-    complete_link(U);
-  }
   // complex component k of the spinor at site d
   __device__ __forceinline__ static f2 comp(const float* f, const float*, int d, int Vb, int k) {
     return ld_comp(f, comp_off<float>(d, Vb, k));
@@ -551,29 +1039,6 @@ struct IO<float> {
 
 template <class S>
 struct IOH {
-  using T = uint4;
-  static constexpr int LINK_U = HGAUGE_NU;
-  static constexpr int CLOV_U = HCLOV_NU;
-  __device__ __forceinline__ static void unpack(const T& t, float* v) { unpack8<S>(t, v); }
-  // chiral block cb: units 4 cb .. 4 cb + 4, offset 4 cb
-  __device__ __forceinline__ static void block_smem(const T* A, int Vh, int h, int cb, float* P) {
-    float v[40];
-#pragma unroll
-    for (int u = 0; u < 5; ++u) unpack(A[(4 * cb + u) * Vh + h], v + 8 * u);
-#pragma unroll
-    for (int k = 0; k < 36; ++k) P[k] = cb ? v[4 + k] : v[k];
-  }
-  __device__ __forceinline__ static void link2_smem(const T* sl, int Vbp, int q, int mu, Link<float>& U) {
-    float v[16];
-    const int u0 = link_unit(mu);
-    unpack(sl[u0 * Vbp + q], v);
-    unpack(sl[(u0 + 1) * Vbp + q], v + 8);
-    link_rows_from16(v, mu, U);
-  }
-  __device__ __forceinline__ static void link_smem(const T* sl, int Vbp, int q, int mu, Link<float>& U) {
-    link2_smem(sl, Vbp, q, mu, U);
-    complete_link(U);
-  }
   // 32-bit word of complex component k: unit k / 4, position k % 4
   __device__ __forceinline__ static size_t word(int d, int Vb, int k) {
     return hunit<HSPIN_NU>(d, Vb, k >> 2) * 4 + (k & 3);
@@ -614,77 +1079,6 @@ struct IO<__half> : IOH<__half> {};
 template <>
 struct IO<__nv_bfloat16> : IOH<__nv_bfloat16> {};
 
-// block sum of three per-thread partials with one barrier: every warp
-// leaves its three warp sums in sh[3 w ..], and after the barrier every warp
-// adds all of them up itself, in the same fixed order, so every thread holds
-// the same bits.  Two calls must be separated by another barrier of the CTA
-// (all reads of one call are done before the next call writes).
-__device__ __forceinline__ void block_sum3_1(float ra, float rb, float rc, float& a, float& b, float& c,
-                                             float* sh) {
-  ra = warp_sum_r<float>(ra);
-  rb = warp_sum_r<float>(rb);
-  rc = warp_sum_r<float>(rc);
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31, nw = blockDim.x >> 5;
-  if (l == 0) { sh[3 * w] = ra; sh[3 * w + 1] = rb; sh[3 * w + 2] = rc; }
-  __syncthreads();
-  const float x = l < nw ? sh[3 * l] : 0.f, y = l < nw ? sh[3 * l + 1] : 0.f, z = l < nw ? sh[3 * l + 2] : 0.f;
-  a = warp_sum_r<float>(x);
-  b = warp_sum_r<float>(y);
-  c = warp_sum_r<float>(z);
-}
-
-// own 3 rows of a staged chiral block (site h) times v6
-template <class S>
-__device__ __forceinline__ void rows3(const typename IO<S>::T* A, int Vh, int h, int cb, int half, const f2 v6[6],
-                                      f2 y[3]) {
-  float P[36];
-  IO<S>::block_smem(A, Vh, h, cb, P);
-  f2 y6[6];
-  herm6<float>(P, v6, y6);
-#pragma unroll
-  for (int i = 0; i < 3; ++i) y[i] = half ? y6[3 + i] : y6[i];
-}
-
-// link mu of local site q from the staged block links, its third row from
-// the rows rebuilt once per sweep (row3[(3 mu + c) Vbp + q])
-template <class S>
-__device__ __forceinline__ void slink(const typename IO<S>::T* sl, const f2* row3, int Vbp, int q, int mu,
-                                      Link<float>& U) {
-  IO<S>::link2_smem(sl, Vbp, q, mu, U);
-#pragma unroll
-  for (int c = 0; c < 3; ++c) U.m[2][c] = row3[(3 * mu + c) * Vbp + q];
-}
-
-// hop_block with the neighbour indices already known (-1: outside the block)
-template <class S>
-__device__ __forceinline__ void hop_block_q(int qf, int qb, const typename IO<S>::T* sl, const f2* row3, const f2* buf,
-                                            int Vbp,
-                                            int Vh, int q, int sub, f2 out[3]) {
-  Spinor<float> acc;
-#pragma unroll
-  for (int k = 0; k < 12; ++k) acc.c[k] = mk(0.f, 0.f);
-  const Dir<float> dr = make_dir<float>(sub);
-  f2 hh[2][3], y[2][3];
-  Spinor<float> nb;
-  if (qf >= 0) {
-    smem_spinor<float>(buf, Vh, qf >= Vh ? qf - Vh : qf, nb);
-    project_rt<float>(nb, dr, -1.f, hh);
-    Link<float> U;
-    slink<S>(sl, row3, Vbp, q, sub, U);
-    su3_mul(U, hh, y);
-    accumulate_rt<float>(acc, y, dr, -1.f, 1.f);
-  }
-  if (qb >= 0) {
-    smem_spinor<float>(buf, Vh, qb >= Vh ? qb - Vh : qb, nb);
-    project_rt<float>(nb, dr, 1.f, hh);
-    Link<float> U;
-    slink<S>(sl, row3, Vbp, qb, sub, U);
-    su3_mul_dag(U, hh, y);
-    accumulate_rt<float>(acc, y, dr, 1.f, 1.f);
-  }
-  reduce_scatter<float>(acc, sub, out);
-}
-
 // own 3 components of the full (global) hopping sum at device site d
 template <class S>
 __device__ __forceinline__ void hop_global_s(const Geom& g, const S* x, const float* xn, const S* gauge, int d,
@@ -716,267 +1110,6 @@ __device__ __forceinline__ void hop_global_s(const Geom& g, const S* x, const fl
     accumulate_rt<float>(acc, y, dr, 1.f, (e & NEG_BIT) ? -1.f : 1.f);
   }
   reduce_scatter<float>(acc, sub, out);
-}
-
-__device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-
-// bn / xn: site norms of b and x (half storage only; ignored for FP32).
-// SM is the type the staged block operators are kept in: the storage type S,
-// or FP32 for half storage (SM = float, S half): the half units are staged
-// into the upper half of each FP32 array and widened in place once per
-// sweep, so that the block solve's many reads of the staged links and
-// clover blocks need no unpacking.
-template <class S, class SM>
-__global__ void __launch_bounds__(512) k_sap_stg(Geom g, int colour, int mr_iters, int x_is_zero,
-                                                 const S* __restrict__ b, const float* __restrict__ bn,
-                                                 S* __restrict__ x, float* __restrict__ xn,
-                                                 const S* __restrict__ gauge, const S* __restrict__ clov,
-                                                 const S* __restrict__ clov_inv, int* status, long long wait_limit) {
-  using T = typename IO<SM>::T;
-  constexpr bool WIDEN = !std::is_same<S, SM>::value;
-  static_assert(sizeof(T) == sizeof(typename IO<S>::T), "16-byte units in both types");
-  constexpr unsigned UB = sizeof(T);            // bytes per unit
-  constexpr int LU = IO<SM>::LINK_U, CU = IO<SM>::CLOV_U;     // staged units per site
-  constexpr int LG = IO<S>::LINK_U, CG = IO<S>::CLOV_U;       // units per site in global memory
-  static_assert(!WIDEN || (LU == 2 * LG && CU == 2 * CG), "a half unit widens into two FP32 units");
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int Vb = g.Vb, Vh = Vb / 2, Vbp = Vb + LPAD;
-  T* sl = reinterpret_cast<T*>(smem_raw);                               // [LU][Vb + LPAD]
-  T* Aee = sl + (size_t)LU * Vbp;                                       // [CU][Vh]
-  T* Aoi = Aee + CU * Vh;                                               // [CU][Vh]
-  f2* E = reinterpret_cast<f2*>(Aoi + CU * Vh);                         // [12][Vh]
-  f2* O = E + 12 * Vh;                                                  // [12][Vh]
-  float* red = reinterpret_cast<float*>(O + 12 * Vh);                   // [3 * warps + 3]
-  f2* row3 = reinterpret_cast<f2*>(red + 200);                          // [12][Vb + LPAD]
-
-  // CTA c handles right-hand side c % nrhs of block c / nrhs of the colour:
-  // the CTAs of one block run side by side, so the block's links and clover
-  // blocks come from DRAM once and from L2 for the other right-hand sides
-  const int nrhs = gridDim.x / (g.nb / 2);
-  const int rhs = blockIdx.x % nrhs;
-  const int B = block_of_colour(g, colour, blockIdx.x / nrhs);
-  const size_t off = (size_t)rhs * g.V * SPINOR_NR;
-  const size_t noff = (size_t)rhs * g.V;
-  b += off;
-  x += off;
-  if (bn) bn += noff;       // site norms exist for half storage only
-  if (xn) xn += noff;
-  const int t = threadIdx.x;
-  const int h = t >> 2, sub = t & 3;
-  const int cb = sub >> 1, half = sub & 1;
-  const int de = B * Vb + h, dO = B * Vb + Vh + h;
-  // block-internal neighbours of this thread's direction, even and odd site
-  const int qf_e = __ldg(g.bnbr + (2 * sub) * Vb + h), qb_e = __ldg(g.bnbr + (2 * sub + 1) * Vb + h);
-  const int qf_o = __ldg(g.bnbr + (2 * sub) * Vb + Vh + h), qb_o = __ldg(g.bnbr + (2 * sub + 1) * Vb + Vh + h);
-
-  // stage the block's links (and A_ee, A_oo^-1) with bulk asynchronous
-  // copies: global unit row u lands in staged row u, or in row LU - LG + u
-  // (CU - CG + u) when it is widened afterwards
-  __shared__ __align__(8) uint64_t mbar;
-  if (t == 0) {
-    mbar_init(&mbar, 1);
-    mbar_fence_init();
-  }
-  __syncthreads();
-  {
-    const unsigned link_row = (unsigned)Vb * UB, half_row = (unsigned)Vh * UB;
-    if (t == 0) mbar_expect_tx(&mbar, (unsigned)LG * link_row + 2u * CG * half_row);
-    __syncthreads();
-    if (t < LG) {
-      const T* src = reinterpret_cast<const T*>(gauge) + (size_t)B * LG * Vb;
-      bulk_g2s(sl + (size_t)(LU - LG + t) * Vbp, src + (size_t)t * Vb, link_row, &mbar);
-    } else if (t < LG + CG) {
-      const int u = t - LG;
-      const T* ca = reinterpret_cast<const T*>(clov) + (size_t)B * CG * Vb;
-      bulk_g2s(Aee + (size_t)(CU - CG + u) * Vh, ca + (size_t)u * Vb, half_row, &mbar);
-    } else if (t < LG + 2 * CG) {
-      const int u = t - LG - CG;
-      const T* ci = reinterpret_cast<const T*>(clov_inv) + (size_t)B * CG * Vb;
-      bulk_g2s(Aoi + (size_t)(CU - CG + u) * Vh, ci + (size_t)u * Vb + Vh, half_row, &mbar);
-    }
-  }
-  // b and x may still be written by the previous kernel of the stream
-  grid_dependency_wait();
-
-  // residual r = b - D x on the own components of both sites: the hops and
-  // the odd site's clover product from global memory while the block is
-  // staged, the even site's clover product from the staged A_ee after it
-  f2 re[3], ro[3], xe6[6];
-#pragma unroll
-  for (int par = 0; par < 2; ++par) {
-    const int d = par ? dO : de;
-    f2 r[3];
-#pragma unroll
-    for (int i = 0; i < 3; ++i) r[i] = IO<S>::comp(b, bn, d, Vb, 3 * sub + i);
-    if (!x_is_zero) {
-      f2 hop[3], x6[6];
-      hop_global_s<S>(g, x, xn, gauge, d, sub, hop);
-#pragma unroll
-      for (int i = 0; i < 6; ++i) x6[i] = IO<S>::comp(x, xn, d, Vb, 6 * cb + i);
-#pragma unroll
-      for (int i = 0; i < 3; ++i) {
-        r[i].re += 0.5f * hop[i].re;
-        r[i].im += 0.5f * hop[i].im;
-      }
-      if (par) {
-        float P[36];
-        IO<S>::block36(clov, d, Vb, cb, P);
-        f2 y6[6];
-        herm6<float>(P, x6, y6);
-#pragma unroll
-        for (int i = 0; i < 3; ++i) r[i] = r[i] - (half ? y6[3 + i] : y6[i]);
-      } else {
-#pragma unroll
-        for (int i = 0; i < 6; ++i) xe6[i] = x6[i];
-      }
-    }
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      if (par) ro[i] = r[i];
-      else re[i] = r[i];
-    }
-  }
-  // the staged block must have landed (bounded wait; on time-out record
-  // DDAMG_ETIMEOUT, wait again for the copies in flight, and leave x alone)
-  {
-    const bool ok = mbar_wait_bounded(&mbar, 0, wait_limit);
-    if (__syncthreads_or(!ok)) {
-      if (t == 0) atomicExch(status, 6);
-      mbar_wait_bounded(&mbar, 0, MBAR_POLL_LIMIT);
-      return;
-    }
-  }
-  if constexpr (WIDEN) {
-    // half unit k of a site (staged row n + k of an array of 2 n rows) holds
-    // the values of FP32 units 2 k and 2 k + 1.  One thread widens one site
-    // of one array in increasing k: the rows 2 k, 2 k + 1 it writes are
-    // half rows n + k' with k' <= k, already read by the same thread, and
-    // no other thread touches the site's column.
-    for (int s = t; s < Vb + 2 * Vh; s += blockDim.x) {
-      T* a;
-      int n, stride, q;
-      if (s < Vb) { a = sl; n = LG; stride = Vbp; q = s; }
-      else if (s < Vb + Vh) { a = Aee; n = CG; stride = Vh; q = s - Vb; }
-      else { a = Aoi; n = CG; stride = Vh; q = s - Vb - Vh; }
-      for (int k = 0; k < n; ++k) {
-        float v[8];
-        unpack8<S>(*reinterpret_cast<const uint4*>(a + (size_t)(n + k) * stride + q), v);
-        a[(size_t)(2 * k) * stride + q] = make_float4(v[0], v[1], v[2], v[3]);
-        a[(size_t)(2 * k + 1) * stride + q] = make_float4(v[4], v[5], v[6], v[7]);
-      }
-    }
-    __syncthreads();
-  }
-  if (!x_is_zero) {     // r_e -= A_ee x_e, A_ee staged
-    f2 ax[3];
-    rows3<SM>(Aee, Vh, h, cb, half, xe6, ax);
-#pragma unroll
-    for (int i = 0; i < 3; ++i) re[i] = re[i] - ax[i];
-  }
-  // the third rows of the staged links, rebuilt once per sweep instead of
-  // at every hop (visible to the hops after the barrier below)
-  for (int k = t; k < 4 * Vb; k += blockDim.x) {
-    const int mu = k / Vb, q = k - mu * Vb;
-    Link<float> U;
-    IO<SM>::link_smem(sl, Vbp, q, mu, U);
-#pragma unroll
-    for (int c = 0; c < 3; ++c) row3[(3 * mu + c) * Vbp + q] = U.m[2][c];
-  }
-  auto ainv_rows = [&](const f2 v6[6], f2 y[3]) { rows3<SM>(Aoi, Vh, h, cb, half, v6, y); };
-  auto aee_rows = [&](const f2 v6[6], f2 y[3]) { rows3<SM>(Aee, Vh, h, cb, half, v6, y); };
-  // u_o = A_oo^-1 r_o
-  {
-    f2 v6[6], u[3];
-    chiral6<float>(ro, sub, v6);
-    ainv_rows(v6, u);
-#pragma unroll
-    for (int i = 0; i < 3; ++i) O[(3 * sub + i) * Vh + h] = u[i];
-  }
-  __syncthreads();
-  // rhs_e = r_e + 1/2 hop(u_o)
-  f2 res[3], xe[3];
-  {
-    f2 tt[3];
-    hop_block_q<SM>(qf_e, qb_e, sl, row3, O, Vbp, Vh, h, sub, tt);
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      res[i] = mk(fmaf(0.5f, tt[i].re, re[i].re), fmaf(0.5f, tt[i].im, re[i].im));
-      xe[i] = mk(0.f, 0.f);
-    }
-  }
-  for (int it = 0; it < mr_iters; ++it) {
-#pragma unroll
-    for (int i = 0; i < 3; ++i) E[(3 * sub + i) * Vh + h] = res[i];
-    // A_ee res needs only this site's res: formed while the barrier waits
-    f2 p[3];
-    {
-      f2 v6[6];
-      chiral6<float>(res, sub, v6);
-      aee_rows(v6, p);
-    }
-    __syncthreads();
-    {  // odd: w = A_oo^-1 (-1/2 hop(res))
-      f2 tt[3], v6[6], w[3];
-      hop_block_q<SM>(qf_o, qb_o, sl, row3, E, Vbp, Vh, Vh + h, sub, tt);
-#pragma unroll
-      for (int i = 0; i < 3; ++i) tt[i] = -0.5f * tt[i];
-      chiral6<float>(tt, sub, v6);
-      ainv_rows(v6, w);
-#pragma unroll
-      for (int i = 0; i < 3; ++i) O[(3 * sub + i) * Vh + h] = w[i];
-    }
-    __syncthreads();
-    float pr_re = 0.f, pr_im = 0.f, pp_r = 0.f;
-    {  // even: p = A_ee res + 1/2 hop(w)
-      f2 tt[3];
-      hop_block_q<SM>(qf_e, qb_e, sl, row3, O, Vbp, Vh, h, sub, tt);
-#pragma unroll
-      for (int i = 0; i < 3; ++i) {
-        p[i] = mk(fmaf(0.5f, tt[i].re, p[i].re), fmaf(0.5f, tt[i].im, p[i].im));
-        pr_re += p[i].re * res[i].re + p[i].im * res[i].im;
-        pr_im += p[i].re * res[i].im - p[i].im * res[i].re;
-        pp_r += p[i].re * p[i].re + p[i].im * p[i].im;
-      }
-    }
-    float dre, dim, pp;
-    block_sum3_1(pr_re, pr_im, pp_r, dre, dim, pp, red);
-    if (pp > 0.f) {
-      const f2 a = mk(dre / pp, dim / pp);
-#pragma unroll
-      for (int i = 0; i < 3; ++i) {
-        fma(xe[i], a, res[i]);
-        res[i] = res[i] - a * p[i];
-      }
-    }
-  }
-  // the next sweep may start its prologue
-  launch_dependents();
-  // e_o = A_oo^-1 (r_o + 1/2 hop(e_e))
-#pragma unroll
-  for (int i = 0; i < 3; ++i) E[(3 * sub + i) * Vh + h] = xe[i];
-  __syncthreads();
-  f2 eo[3];
-  {
-    f2 tt[3], v6[6];
-    hop_block_q<SM>(qf_o, qb_o, sl, row3, E, Vbp, Vh, Vh + h, sub, tt);
-#pragma unroll
-    for (int i = 0; i < 3; ++i) tt[i] = mk(fmaf(0.5f, tt[i].re, ro[i].re), fmaf(0.5f, tt[i].im, ro[i].im));
-    chiral6<float>(tt, sub, v6);
-    ainv_rows(v6, eo);
-  }
-  f2 ve[3], vo[3];
-#pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    ve[i] = xe[i];
-    vo[i] = eo[i];
-    if (!x_is_zero) {
-      ve[i] = ve[i] + IO<S>::comp(x, xn, de, Vb, 3 * sub + i);
-      vo[i] = vo[i] + IO<S>::comp(x, xn, dO, Vb, 3 * sub + i);
-    }
-  }
-  IO<S>::store3(x, xn, de, Vb, sub, ve);
-  IO<S>::store3(x, xn, dO, Vb, sub, vo);
 }
 
 // ---------------------------------------------------------------------------
@@ -1033,85 +1166,75 @@ size_t sap_smem_bytes(const Geom& g, int real_size) {
   return units * 16 + bufs + 100 * sizeof(double);
 }
 
-// shared memory of the staged kernel: link rows (LU units per site, padded),
-// the even half of A and the odd half of A^-1 (CU units per site each), the
-// even and odd work vectors, the reduction slots and the third rows of the
-// staged links; 16-byte units
-static size_t sap_stg_smem(const Geom& g, int LU, int CU) {
-  const int Vh = g.Vb / 2;
-  size_t bytes = (size_t)LU * (g.Vb + LPAD) * 16;
-  bytes += (size_t)2 * CU * Vh * 16;
-  bytes += (size_t)24 * Vh * 8;
-  bytes += 100 * sizeof(double);
-  bytes += (size_t)12 * (g.Vb + LPAD) * 8;     // third link rows (FP32 complex)
-  return bytes;
+// shared memory of the block kernel: published spinors and half spinors sent
+// ahead, the reduction slots, and the staged operators or, once these are in
+// registers, the kept vectors, x, b or the residual, and the messages
+static size_t sap_block_smem(const Geom& g, int LU, int CU) {
+  const size_t Vh = g.Vb / 2, ops = (size_t)LU * g.Vb * 16 + (size_t)2 * CU * Vh * 16;
+  const size_t after = ((size_t)18 * g.Vb + blk::msg_units(g)) * 16;
+  return 36 * (Vh + 1) * 16 + 16 * (Vh / 32) + (ops > after ? ops : after);
 }
 
-static bool sap_stg_ok(const Geom& g, int LU, int CU) {
-  const int Vh = g.Vb / 2;
-  return Vh % 32 == 0 && 4 * Vh <= 512 && sap_stg_smem(g, LU, CU) <= 226 * 1024;
+bool sap_block_ok(const Geom& g) { return g.Vb % 64 == 0 && g.Vb <= 256; }
+size_t sap_res_bytes(const Geom& g) { return (size_t)g.V / 2 * 96; }
+size_t sap_msg_bytes(const Geom& g) {      // 48 bytes per site of each of a block's eight faces
+  size_t sites = 0;
+  for (int mu = 0; mu < 4; ++mu) sites += 2 * (size_t)(g.Vb / g.b[mu]);
+  return (size_t)g.nb * sites * 48;
 }
 
-bool sap_half_ok(const Geom& g) { return sap_stg_ok(g, HGAUGE_NU, HCLOV_NU); }
-bool sap_staged_ok(const Geom& g) { return sap_stg_ok(g, 12, 18); }
-
-template <class S, class SM>
-static cudaError_t launch_stg(const Geom& g, int colour, int mr_iters, bool x_is_zero, const S* b, const float* bn,
-                              S* x, float* xn, const S* gauge, const S* clover, const S* clover_inv, int nrhs,
-                              int* status, long long wait_limit, cudaStream_t st) {
-  const size_t need = sap_stg_smem(g, stg::IO<SM>::LINK_U, stg::IO<SM>::CLOV_U);
-  {
-    // the attribute is per device and per instance; set it on every launch
-    // whose size exceeds what this device's instance was given
-    static std::mutex mu;
-    static size_t cfg[64] = {};
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    std::lock_guard<std::mutex> lock(mu);
-    if (cfg[dev] < need) {
-      cudaError_t e =
-          cudaFuncSetAttribute(stg::k_sap_stg<S, SM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need);
-      if (e != cudaSuccess) return e;
-      cfg[dev] = need;
+template <class S, int VB>
+static cudaError_t launch_block(const Geom& g, const blk::SapArgs& args, cudaStream_t st, bool overlap) {
+  const size_t need = sap_block_smem(g, blk::Ops<S>::LU, blk::Ops<S>::CU);
+  cudaError_t e = raise_smem_limit((const void*)blk::k_sap_block<S, VB>, need);
+  if (e != cudaSuccess) return e;
+  int dev = 0, sms = 0;
+  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+  // right-hand sides per CTA: a CTA loads its block's operators once for all
+  // of them (about a quarter of a right-hand side's time), but few CTAs of
+  // many right-hand sides leave SMs idle in the last wave
+  blk::SapArgs a = args;
+  const long long slots = (long long)sms * (256 / g.Vb), blocks = g.nb / 2;
+  double best = 0.0;
+  for (int slices = 1; slices <= a.nrhs; ++slices) {
+    const int per = (a.nrhs + slices - 1) / slices;
+    if ((a.nrhs + per - 1) / per != slices) continue;
+    const double cost = (double)((blocks * slices + slots - 1) / slots) * (per + 0.25);
+    if (slices == 1 || cost < best) {
+      best = cost;
+      a.per = per;
     }
   }
   cudaLaunchConfig_t lc = {};
-  lc.gridDim = dim3((unsigned)(g.nb / 2) * (unsigned)nrhs);
-  lc.blockDim = dim3(2 * g.Vb);
+  lc.gridDim = dim3((unsigned)(blocks * ((a.nrhs + a.per - 1) / a.per)));
+  lc.blockDim = dim3(g.Vb);
   lc.dynamicSmemBytes = need;
   lc.stream = st;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // prologue overlaps the previous kernel
   at[0].val.programmaticStreamSerializationAllowed = 1;
   lc.attrs = at;
-  lc.numAttrs = 1;
-  const int zero = x_is_zero ? 1 : 0;
-  cudaError_t e = cudaLaunchKernelEx(&lc, stg::k_sap_stg<S, SM>, g, colour, mr_iters, zero, b, bn, x, xn, gauge,
-                                     clover, clover_inv, status, wait_limit);
+  lc.numAttrs = overlap ? 1 : 0;
+  e = cudaLaunchKernelEx(&lc, blk::k_sap_block<S, VB>, a);
   ++g_launches;
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-template <class S>
-cudaError_t sap_sweep_h(const Geom& g, int colour, int mr_iters, bool x_is_zero, const void* b, const float* bn,
-                        void* x, float* xn, const void* gauge, const void* clover, const void* clover_inv, int nrhs,
-                        int* status, long long wait_limit, cudaStream_t st, bool widen) {
-  if (!sap_half_ok(g)) return cudaErrorInvalidValue;
-  if (widen && sap_staged_ok(g))
-    return launch_stg<S, float>(g, colour, mr_iters, x_is_zero, static_cast<const S*>(b), bn, static_cast<S*>(x), xn,
-                                static_cast<const S*>(gauge), static_cast<const S*>(clover),
-                                static_cast<const S*>(clover_inv), nrhs, status, wait_limit, st);
-  return launch_stg<S, S>(g, colour, mr_iters, x_is_zero, static_cast<const S*>(b), bn, static_cast<S*>(x), xn,
-                          static_cast<const S*>(gauge), static_cast<const S*>(clover),
-                          static_cast<const S*>(clover_inv), nrhs, status, wait_limit, st);
+cudaError_t sap_block_sweep(const Geom& g, int half_kind, int colour, int mr_iters, const SapStep& step, const float* b,
+                            float* x, void* res, void* msg, const void* gauge, const void* clover,
+                            const void* clover_inv, int nrhs, int* status, long long wait_limit, cudaStream_t st) {
+  if (!sap_block_ok(g)) return cudaErrorInvalidValue;
+  blk::SapArgs a{g, colour, mr_iters, nrhs, nrhs, step.first, step.take, step.give, step.keep, b, x,
+                 static_cast<float4*>(res), static_cast<float4*>(msg), gauge, clover, clover_inv, status, wait_limit};
+  auto launch = [&](auto vb) -> cudaError_t {
+    constexpr int VB = decltype(vb)::value;
+    if (half_kind == 0) return launch_block<__half, VB>(g, a, st, step.overlap);
+    if (half_kind == 1) return launch_block<__nv_bfloat16, VB>(g, a, st, step.overlap);
+    return launch_block<float, VB>(g, a, st, step.overlap);
+  };
+  return g.Vb == 256 ? launch(std::integral_constant<int, 256>{}) : launch(std::integral_constant<int, 0>{});
 }
-template cudaError_t sap_sweep_h<__half>(const Geom&, int, int, bool, const void*, const float*, void*, float*,
-                                         const void*, const void*, const void*, int, int*, long long, cudaStream_t,
-                                         bool);
-template cudaError_t sap_sweep_h<__nv_bfloat16>(const Geom&, int, int, bool, const void*, const float*, void*,
-                                                float*, const void*, const void*, const void*, int, int*, long long,
-                                                cudaStream_t, bool);
 
 template <class S>
 cudaError_t dslash4(const Geom& g, const void* x, const float* xn, void* y, float* yn, const void* gauge,
@@ -1133,14 +1256,8 @@ template cudaError_t dslash4<__nv_bfloat16>(const Geom&, const void*, const floa
 
 template <class R>
 cudaError_t sap_sweep(const Geom& g, int colour, int mr_iters, bool x_is_zero, const R* b, R* x,
-                      const R* gauge, const R* clover, const R* clover_inv, int nrhs, int* status,
-                      long long wait_limit, cudaStream_t st, bool staged) {
-  if constexpr (sizeof(R) == 4) {
-    if (staged && sap_stg_ok(g, 12, 18)) {
-      return launch_stg<float, float>(g, colour, mr_iters, x_is_zero, b, nullptr, x, nullptr, gauge, clover,
-                                      clover_inv, nrhs, status, wait_limit, st);
-    }
-  }
+                      const R* gauge, const R* clover, const R* clover_inv, int nrhs,
+                      cudaStream_t st) {
   int threads = sap_threads(g);
   size_t smem = sap_smem_bytes(g, sizeof(R));
   {
@@ -1164,9 +1281,8 @@ cudaError_t sap_sweep(const Geom& g, int colour, int mr_iters, bool x_is_zero, c
 }
 
 template cudaError_t sap_sweep<float>(const Geom&, int, int, bool, const float*, float*, const float*,
-                                      const float*, const float*, int, int*, long long, cudaStream_t, bool);
+                                      const float*, const float*, int, cudaStream_t);
 template cudaError_t sap_sweep<double>(const Geom&, int, int, bool, const double*, double*,
-                                       const double*, const double*, const double*, int, int*, long long,
-                                       cudaStream_t, bool);
+                                       const double*, const double*, const double*, int, cudaStream_t);
 
 }  // namespace ddamg
