@@ -693,16 +693,16 @@ __host__ __device__ __forceinline__ int msg_units(const Geom& g) {
   return 6 * (g.Vb / g.b[0] + g.Vb / g.b[1] + g.Vb / g.b[2] + g.Vb / g.b[3]);
 }
 
-// VB: the block's sites if known at compile time (4^4 blocks: constant strides
-// take 10 % off the solve), else 0
+// VB: the block's sites (constant strides take 10 % off the solve)
 template <class S, int VB>
-__global__ void __launch_bounds__(256, 1) k_sap_block(SapArgs a) {
+__global__ void __launch_bounds__(VB, 256 / VB) k_sap_block(SapArgs a) {
   using T = typename Ops<S>::T;
   constexpr int LU = Ops<S>::LU, CU = Ops<S>::CU;
   constexpr unsigned UB = sizeof(T);
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const Geom& g = a.g;
-  const int Vb = VB ? VB : g.Vb, Vh = Vb / 2, row = Vh + 1, S3 = msg_units(g);
+  constexpr int Vb = VB, Vh = Vb / 2, row = Vh + 1;
+  const int S3 = msg_units(g);
   float4* pub = reinterpret_cast<float4*>(smem_raw);       // [parity][6][Vh + 1] published spinors
   float4* gx = pub + 12 * row;                             // [parity][12][Vh + 1] sent ahead
   float4* red = gx + 24 * row;                             // [warps of one parity]
@@ -1233,7 +1233,12 @@ cudaError_t sap_block_sweep(const Geom& g, int half_kind, int colour, int mr_ite
     if (half_kind == 1) return launch_block<__nv_bfloat16, VB>(g, a, st, step.overlap);
     return launch_block<float, VB>(g, a, st, step.overlap);
   };
-  return g.Vb == 256 ? launch(std::integral_constant<int, 256>{}) : launch(std::integral_constant<int, 0>{});
+  switch (g.Vb) {
+    case 64: return launch(std::integral_constant<int, 64>{});
+    case 128: return launch(std::integral_constant<int, 128>{});
+    case 192: return launch(std::integral_constant<int, 192>{});
+    default: return launch(std::integral_constant<int, 256>{});
+  }
 }
 
 template <class S>
