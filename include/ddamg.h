@@ -358,9 +358,7 @@ DDAMG_API ddamg_status ddamg_get_coarse_plan(ddamg_handle h, int nrhs, ddamg_coa
  * problem, the variants' mean times in microseconds and the choice.
  * Variants so far: the Wilson-clover D with one thread per site (0) or four
  * threads per site, one hop direction each (1), in FP32 and in BF16/FP16
- * storage; the coarse GMRES's block products for eight right-hand sides in
- * lockstep with the blocks streamed through shared memory, on the CUDA
- * cores (0) or the tensor cores (1, 3xTF32) ("coarse product"); the FP32
+ * storage; the FP32
  * Schwarz sweep with the block's links and clover blocks in registers and the
  * residual carried between sweeps (0) or by the general kernel (1) ("SAP
  * fp32"; the half-storage sweep has one form); the
@@ -376,8 +374,8 @@ typedef struct {
 } ddamg_tuning;
 DDAMG_API int ddamg_tuning_count(void);
 DDAMG_API ddamg_status ddamg_get_tuning(int i, ddamg_tuning *out);
-/* Use `variant` of the named kernel ("D fp32", "D bf16", "D fp16", "coarse
- * product", "SAP fp32", "SAP bf16", "SAP fp16", "coarse stencil") for every
+/* Use `variant` of the named kernel ("D fp32", "D bf16", "D fp16", "SAP
+ * fp32", "coarse stencil"; a name without variants changes nothing) for every
  * problem instead of the measured choice (variant < 0: measure again);
  * process-wide, for reproducible runs and for checking each variant. */
 DDAMG_API ddamg_status ddamg_pin_variant(const char *kernel, int variant);

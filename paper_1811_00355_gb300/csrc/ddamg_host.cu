@@ -853,22 +853,6 @@ ddamg_status op_coarse_solve(ddamg_ctx* h, const R* bc, R* xc, int nf, double to
   a.restart = h->p.coarse_restart;
   a.max_iter = h->p.coarse_max_iter;
   a.wait_limit = h->wait_grid;
-  if (sizeof(R) == 4) {
-    // eight right-hand sides through the block ring: the block products on
-    // the CUDA cores (0) or the tensor cores (1), the faster one measured on
-    // this call's data the first time (iteration counters left alone)
-    const CoarsePlan pl = coarse_gmres_plan<R>(h->g, h->p.n_v, h->p.coarse_restart, nf);
-    if (pl.ring && pl.NR == 8) {
-      auto run = [&](int var) -> cudaError_t {
-        CoarseSolveArgs t = a;
-        t.tc = var;
-        return coarse_gmres<R>(h->g, t, bc, xc, nf, h->cwork, nullptr, nullptr, h->d_status, h->st);
-      };
-      char key[96];
-      snprintf(key, sizeof key, "coarse %d sites n_v %d fp32 nrhs %d", h->g.nb, h->p.n_v, nf);
-      TRY(tuned(h, "coarse product", key, 2, run, &a.tc));
-    }
-  }
   addf(h, nf * flops_coarse_fixed(h));   // iterations are added when their counts are read
   CK(timed(h, 2, [&] {
     return coarse_gmres<R>(h->g, a, bc, xc, nf, h->cwork, iters_dev, h->d_iters_acc, h->d_status, h->st);
@@ -2373,7 +2357,8 @@ ddamg_status coarse_solve_noalloc_impl(ddamg_ctx* h, int nrhs, const double* in,
                                        int* iters) {
   const size_t nc = (size_t)nrhs * h->g.nb * h->n2;
   const size_t vec = (nc * 2 * sizeof(R) + 255) / 256 * 256;
-  const CoarsePlan plan = coarse_gmres_plan<R>(h->g, h->p.n_v, h->p.coarse_restart, nrhs);
+  // (the form that keeps its basis in shared memory where it can: least scratch)
+  const CoarsePlan plan = coarse_gmres_plan<R>(h->g, h->p.n_v, h->p.coarse_restart, nrhs, false);
   const size_t work = plan.work_bytes;
   if (work == 0) return fail(h, DDAMG_EINVAL, "no launch configuration for the coarse solve");
   const size_t need = 2 * vec + work;
@@ -2395,6 +2380,7 @@ ddamg_status coarse_solve_noalloc_impl(ddamg_ctx* h, int nrhs, const double* in,
   a.restart = h->p.coarse_restart;
   a.max_iter = h->p.coarse_max_iter;
   a.wait_limit = h->wait_grid;
+  a.wide = 0;
   CK(coarse_from_f64<R>(in, bin, nc, h->st));
   CK(coarse_gmres<R>(h->g, a, bin, xout, nrhs, wk, h->d_iters, nullptr, h->d_status, h->st, &plan));
   CK(coarse_to_f64<R>(xout, out, nc, h->st));

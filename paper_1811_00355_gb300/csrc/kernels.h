@@ -311,7 +311,7 @@ struct CoarseSolveArgs {
   int restart;      // <= 64
   int max_iter;
   long long wait_limit;   // polls of a grid-barrier wait before it gives up (DDAMG_ETIMEOUT)
-  int tc = 0;             // eight right-hand sides through the block ring: products on the tensor cores
+  int wide = 1;           // the form for many right-hand sides where it applies (its basis in global scratch)
 };
 // launch configuration of the coarse GMRES for nrhs right-hand sides (all
 // zero if none exists): NR right-hand sides in lockstep per launch pass, G
@@ -332,7 +332,7 @@ struct CoarsePlan {
   size_t smem_bytes, work_bytes;
 };
 template <class R>
-CoarsePlan coarse_gmres_plan(const Geom& g, int n, int restart, int nrhs);
+CoarsePlan coarse_gmres_plan(const Geom& g, int n, int restart, int nrhs, bool wide = true);
 size_t coarse_gmres_work_bytes(const Geom& g, int n, int restart, int real_size);
 // bytes of `work` that coarse_gmres() touches for nrhs right-hand sides (0 if
 // no launch configuration exists)

@@ -22,9 +22,9 @@
 #include <algorithm>
 #include <mutex>
 
+#include "cgmres.cuh"
 #include "common.cuh"
 #include "kernels.h"
-#include "mma_tf32.cuh"
 
 namespace ddamg {
 
@@ -47,93 +47,6 @@ constexpr int NRMAX = 12;
 constexpr int RING = 4;
 constexpr int RING_MIN_N2 = 32;
 
-__device__ __forceinline__ cpx<float> ldc(const cpx<float>* p) {
-  float2 t = __ldcg(reinterpret_cast<const float2*>(p));
-  return mk(t.x, t.y);
-}
-__device__ __forceinline__ cpx<double> ldc(const cpx<double>* p) {
-  double2 t = __ldcg(reinterpret_cast<const double2*>(p));
-  return mk(t.x, t.y);
-}
-
-template <class T>
-__device__ __forceinline__ T wsum(T v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
-// Grid barrier on a counter that only grows during a launch (zeroed before
-// it): at its e-th barrier every CTA adds 1 and waits until the counter
-// reaches e * gridDim.x.  The arrival is a fence followed by a relaxed
-// reduction (no reply awaited), the wait an acquire load, so a barrier costs
-// about one L2 round trip after the last arrival.  The wait is bounded (about
-// a second); on time-out the CTA records DDAMG_ETIMEOUT and leaves, and the
-// CTAs still waiting for it then time out at this or their next barrier.
-__device__ unsigned ld_acquire_gpu(const unsigned* p) {
-  unsigned v;
-  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-  return v;
-}
-
-__shared__ unsigned bar_epoch;       // barriers passed by this CTA in this launch
-
-// thread 0 zeroes the count at kernel entry (a __syncthreads must follow
-// before the first barrier)
-__device__ void grid_barrier_reset() {
-  if (threadIdx.x == 0) bar_epoch = 0;
-}
-
-// Split form: grid_arrive publishes this CTA's writes and counts it in;
-// grid_wait returns once every CTA has arrived.  Between the two a CTA may do
-// work that touches only its own shared memory and registers.
-__device__ void grid_arrive(unsigned* bar) {
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    ++bar_epoch;
-    __threadfence();                 // the CTA's writes (ordered by the bar.sync above) first
-    asm volatile("red.relaxed.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
-  }
-}
-
-__device__ bool grid_wait(unsigned* bar, int* status, long long limit) {
-  __shared__ int ok_s;
-  if (threadIdx.x == 0) {
-    const unsigned target = bar_epoch * gridDim.x;
-    int ok = 1;
-    long long spins = 0;
-    while ((int)(ld_acquire_gpu(bar) - target) < 0) {
-      if (++spins > limit) {
-        atomicExch(status, 6);
-        ok = 0;
-        break;
-      }
-    }
-    ok_s = ok;
-  }
-  __syncthreads();
-  return ok_s != 0;
-}
-
-__device__ bool grid_barrier(unsigned* bar, int* status, long long limit) {
-  grid_arrive(bar);
-  return grid_wait(bar, status, limit);
-}
-
-// L2 prefetch of `bytes` bytes at p (16-byte aligned, a multiple of 16) by
-// the calling warp, in bulk prefetches of at most 32 KB per lane: the block
-// operators of the next coarse site travel from HBM while this site's block
-// product runs
-__device__ __forceinline__ void prefetch_l2(const void* p, size_t bytes) {
-  constexpr size_t PIECE = 32768;
-  for (size_t off = (size_t)(threadIdx.x & 31) * PIECE; off < bytes; off += 32 * PIECE) {
-    const size_t n = bytes - off < PIECE ? bytes - off : PIECE;
-    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(static_cast<const char*>(p) + off),
-                 "r"((unsigned)n)
-                 : "memory");
-  }
-}
-
 // shared-memory plan, identical on host and device
 struct Plan {
   size_t V, x, rl, w, sv, mvp, tmp;                                    // cpx offsets (bytes)
@@ -146,7 +59,6 @@ struct Plan {
   size_t local_bytes;  // V + x + rl + w (moved to global when too large)
 };
 
-__host__ __device__ inline size_t al16(size_t v) { return (v + 15) / 16 * 16; }
 
 __host__ __device__ inline Plan make_plan(int NR, int L, int n2, int m, int rs, bool local_in_smem,
                                           bool resident = false, bool ring = false) {
@@ -215,7 +127,6 @@ struct CGA {
   int local_in_smem;
   int resident;      // the CTA keeps its even site's D_c blocks in shared memory
   int ring;          // block operators streamed through the shared-memory ring
-  int tc;            // ring products of eight right-hand sides on the tensor cores
   cpx<R>* wg;        // [NR][NE][n2]
   cpx<R>* to;        // [NR][NE][n2]
   cpx<R>* xg;        // [NR][NE][n2]
@@ -452,26 +363,6 @@ __global__ void __launch_bounds__(TPB) k_cgmres(CGA<R> a) {
       const int j = tx % NP, rest = tx / NP, rs = rest % RS, cc = rest / RS;
       const int c0 = cc * CW, c1 = min(n2, c0 + CW);
       const cpx<R>* svr = sv + (size_t)rs * NRS * 9 * svs;
-      // Eight right-hand sides on the tensor cores (3xTF32, FP32 accuracy):
-      // per site C' (16 x n2) = A' (16 x 2K) B (2K x n2), with A' rows
-      // m = r + 8 p the real (p = 0) and imaginary (p = 1) rows of the
-      // staged vectors and B the raw blocks.  In a k-step of four complex
-      // columns c0 .. c0 + 3, lane t's k = t and k = t + 4 stand for the real
-      // and imaginary parts of column c0 + t, so for v = sv[r][d][c0 + t]
-      //   A'[r][t] = v.re, A'[r][t + 4] = -v.im, A'[r + 8][t] = v.im, A'[r + 8][t + 4] = v.re
-      // and (b0, b1) = M_d[n0 + g][c0 + t] (one 8-byte load).  Warp (kg, ng)
-      // takes k-steps 2 kg, 2 kg + 1 of every block and n-tiles
-      // ng TPW .. ng TPW + TPW - 1; each block's products go to fresh
-      // accumulators added in FP32, the k-groups' partials meet in mvp.
-      constexpr int TPWMAX = 4;
-      const int NT = n2 / 8, KG = n2 / 8;      // n-tiles; k-groups of two k-steps (n2 / 4 k-steps a block)
-      const int NGR = min(NT, NW / (KG > 0 ? KG : 1));
-      const int TPW = NGR > 0 ? (NT + NGR - 1) / NGR : 0;
-      const bool tc = a.tc && NR == 8 && n2 % 8 == 0 && NGR >= 1 && TPW <= TPWMAX;
-      const int gq = lane >> 2, tq = lane & 3;
-      const int kg = wid % (KG > 0 ? KG : 1), ng = wid / (KG > 0 ? KG : 1);
-      const bool mw = tc && ng < NGR;
-      float* mvpf = reinterpret_cast<float*>(mvp);
       for (int si = 0; si < nsites; ++si) {
         // a site's nd blocks are contiguous: the next site's go to L2 now
         if (si + 1 < nsites && tx < 32) prefetch_l2(blk((unsigned)((si + 1) * nd)), (size_t)nd * bytes);
@@ -481,11 +372,6 @@ __global__ void __launch_bounds__(TPB) k_cgmres(CGA<R> a) {
         for (int r = 0; r < NRS; ++r)
 #pragma unroll
           for (int q = 0; q < RPU; ++q) acc[r][q] = mk(R(0), R(0));
-        float tacc[TPWMAX][4];
-#pragma unroll
-        for (int i = 0; i < TPWMAX; ++i)
-#pragma unroll
-          for (int e = 0; e < 4; ++e) tacc[i][e] = 0.f;
         for (int t = 0; t < nd; ++t) {
           const unsigned b = base + (unsigned)(si * nd + t);
           const bool ok = mbar_wait_bounded(&ring_full[b % RING], (b / RING) & 1u, a.spin_limit);
@@ -499,37 +385,7 @@ __global__ void __launch_bounds__(TPB) k_cgmres(CGA<R> a) {
           }
           if (tx == 0)
             for (; ring_issued < end && ring_issued < b + RING; ++ring_issued) issue(ring_issued);
-          if (tc) {
-            if (mw) {
-              const float* slot = reinterpret_cast<const float*>(ringbuf + (size_t)(b % RING) * nn);
-              const int d = d0 + t;
-              float part[TPWMAX][4];
-#pragma unroll
-              for (int i = 0; i < TPWMAX; ++i)
-#pragma unroll
-                for (int e = 0; e < 4; ++e) part[i][e] = 0.f;
-#pragma unroll
-              for (int h = 0; h < 2; ++h) {
-                const int c = 4 * (2 * kg + h) + tq;
-                const cpx<R> v = sv[(size_t)(gq * 9 + d) * svs + c];
-                const float af[4] = {v.re, v.im, -v.im, v.re};
-                const Split<4> as = split_frag<4>(af);
-#pragma unroll
-                for (int i = 0; i < TPWMAX; ++i) {
-                  const int nt = ng * TPW + i;
-                  if (i < TPW && nt < NT) {
-                    const float2 mv = *reinterpret_cast<const float2*>(slot + ((size_t)c * n2 + nt * 8 + gq) * 2);
-                    const float bv[2] = {mv.x, mv.y};
-                    mma3(part[i], as, split_frag<2>(bv));
-                  }
-                }
-              }
-#pragma unroll
-              for (int i = 0; i < TPWMAX; ++i)
-#pragma unroll
-                for (int e = 0; e < 4; ++e) tacc[i][e] += part[i][e];
-            }
-          } else if (tx < units) {
+          if (tx < units) {
             const T* col = reinterpret_cast<const T*>(ringbuf + (size_t)(b % RING) * nn) + j;
             const int d = d0 + t;
 #pragma unroll 4
@@ -545,39 +401,17 @@ __global__ void __launch_bounds__(TPB) k_cgmres(CGA<R> a) {
             }
           }
         }
-        if (tc) {
-          if (mw)
+        if (tx < units)
 #pragma unroll
-            for (int i = 0; i < TPWMAX; ++i) {
-              const int nt = ng * TPW + i;
-              if (i < TPW && nt < NT)
+          for (int r = 0; r < NRS; ++r)
 #pragma unroll
-                for (int e = 0; e < 4; ++e)
-                  mvpf[((size_t)kg * 16 + gq + (e >= 2 ? 8 : 0)) * n2 + nt * 8 + 2 * tq + (e & 1)] = tacc[i][e];
-            }
-          __syncthreads();
-          for (int idx = tx; idx < NR * n2; idx += TPB) {
-            const int r = idx / n2, row = idx - r * n2;
-            float re = 0.f, im = 0.f;
-            for (int q = 0; q < KG; ++q) {
-              re += mvpf[((size_t)q * 16 + r) * n2 + row];
-              im += mvpf[((size_t)q * 16 + 8 + r) * n2 + row];
-            }
-            emit(si, r, row, mk(re, im));
-          }
-        } else {
-          if (tx < units)
-#pragma unroll
-            for (int r = 0; r < NRS; ++r)
-#pragma unroll
-              for (int q = 0; q < RPU; ++q) mvp[((size_t)cc * NR + rs * NRS + r) * n2 + RPU * j + q] = acc[r][q];
-          __syncthreads();
-          for (int idx = tx; idx < NR * n2; idx += TPB) {
-            const int r = idx / n2, row = idx - r * n2;
-            cpx<R> sum = mk(R(0), R(0));
-            for (int q = 0; q < CC; ++q) sum = sum + mvp[((size_t)q * NR + r) * n2 + row];
-            emit(si, r, row, sum);
-          }
+            for (int q = 0; q < RPU; ++q) mvp[((size_t)cc * NR + rs * NRS + r) * n2 + RPU * j + q] = acc[r][q];
+        __syncthreads();
+        for (int idx = tx; idx < NR * n2; idx += TPB) {
+          const int r = idx / n2, row = idx - r * n2;
+          cpx<R> sum = mk(R(0), R(0));
+          for (int q = 0; q < CC; ++q) sum = sum + mvp[((size_t)q * NR + r) * n2 + row];
+          emit(si, r, row, sum);
         }
         __syncthreads();
       }
@@ -1096,6 +930,7 @@ struct Choice {
   Plan plan;
   bool resident;
   bool ring;
+  WideChoice wide{};      // NR > 0: the kernel for many right-hand sides
 };
 
 // Host state of the launch configurations: the dynamic shared-memory limit
@@ -1132,12 +967,12 @@ cudaError_t smem_attr_locked(int dev, int NR, size_t bytes) {
 inline int first_nr(int nrhs) { return nrhs >= 12 ? 12 : nrhs >= 8 ? 8 : nrhs >= 4 ? 4 : nrhs >= 2 ? 2 : 1; }
 
 template <class R>
-Choice choose_uncached(int dev, const Geom& g, int n2, int m, int nrhs);
+Choice choose_uncached(int dev, const Geom& g, int n2, int m, int nrhs, bool wide);
 
 // launch configurations are cached: the occupancy queries behind them cost
 // far more host time than a coarse solve's launch
 template <class R>
-Choice choose(const Geom& g, int n2, int m, int nrhs) {
+Choice choose(const Geom& g, int n2, int m, int nrhs, bool wide) {
   struct Entry {
     int dev, nb, n2, m, first;
     Choice c;
@@ -1146,20 +981,34 @@ Choice choose(const Geom& g, int n2, int m, int nrhs) {
   static int used = 0;
   int dev = 0;
   cudaGetDevice(&dev);
-  const int first = first_nr(nrhs);
+  // right-hand-side counts that lead to the same choice share an entry
+  const int first = first_nr(nrhs) + (wide ? 16 : 0) + (nrhs >= 5 ? 32 : 0) + (nrhs > 8 ? 64 : 0);
   std::lock_guard<std::mutex> lock(g_cfg_mu);
   for (int i = 0; i < used; ++i) {
     const Entry& e = cache[i];
     if (e.dev == dev && e.nb == g.nb && e.n2 == n2 && e.m == m && e.first == first) return e.c;
   }
-  Choice c = choose_uncached<R>(dev, g, n2, m, nrhs);
+  Choice c = choose_uncached<R>(dev, g, n2, m, nrhs, wide);
   Entry e{dev, g.nb, n2, m, first, c};
   cache[used < 16 ? used++ : (dev + g.nb + first) % 16] = e;
   return c;
 }
 
 template <class R>
-Choice choose_uncached(int dev, const Geom& g, int n2, int m, int nrhs) {
+Choice choose_uncached(int dev, const Geom& g, int n2, int m, int nrhs, bool wide) {
+  if (sizeof(R) == 4 && wide) {
+    const WideChoice w = cgmres_wide_choose(dev, g, n2, m, nrhs);
+    if (w.NR) {
+      Choice c{};
+      c.NR = w.NR;
+      c.G = w.G;
+      c.per = w.per;
+      c.ring = true;
+      c.plan.bytes = w.smem_bytes;
+      c.wide = w;
+      return c;
+    }
+  }
   int sms = 0;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int NE = g.nb / 2;
@@ -1206,10 +1055,10 @@ Choice choose_uncached(int dev, const Geom& g, int n2, int m, int nrhs) {
 }  // namespace
 
 template <class R>
-CoarsePlan coarse_gmres_plan(const Geom& g, int n, int restart, int nrhs) {
+CoarsePlan coarse_gmres_plan(const Geom& g, int n, int restart, int nrhs, bool wide) {
   CoarsePlan out{};
   if (restart > MAXM || restart < 1 || nrhs < 1) return out;
-  Choice ch = choose<R>(g, 2 * n, restart, nrhs);
+  Choice ch = choose<R>(g, 2 * n, restart, nrhs, wide);
   if (ch.NR == 0) return out;
   out.NR = ch.NR;
   out.G = ch.G;
@@ -1218,6 +1067,10 @@ CoarsePlan coarse_gmres_plan(const Geom& g, int n, int restart, int nrhs) {
   out.resident = ch.resident ? 1 : 0;
   out.ring = ch.ring ? 1 : 0;
   out.smem_bytes = ch.plan.bytes;
+  if (ch.wide.NR) {
+    out.work_bytes = ch.wide.work_bytes;
+    return out;
+  }
   // the layout of coarse_gmres() below
   const size_t NE = g.nb / 2, n2 = 2 * n;
   size_t bytes = al16(3 * (size_t)NRMAX * NE * n2 * sizeof(cpx<R>));
@@ -1227,12 +1080,12 @@ CoarsePlan coarse_gmres_plan(const Geom& g, int n, int restart, int nrhs) {
   out.work_bytes = bytes;
   return out;
 }
-template CoarsePlan coarse_gmres_plan<float>(const Geom&, int, int, int);
-template CoarsePlan coarse_gmres_plan<double>(const Geom&, int, int, int);
+template CoarsePlan coarse_gmres_plan<float>(const Geom&, int, int, int, bool);
+template CoarsePlan coarse_gmres_plan<double>(const Geom&, int, int, int, bool);
 
 template <class R>
 size_t coarse_gmres_exact_bytes(const Geom& g, int n, int restart, int nrhs) {
-  return coarse_gmres_plan<R>(g, n, restart, nrhs).work_bytes;
+  return coarse_gmres_plan<R>(g, n, restart, nrhs, true).work_bytes;
 }
 template size_t coarse_gmres_exact_bytes<float>(const Geom&, int, int, int);
 template size_t coarse_gmres_exact_bytes<double>(const Geom&, int, int, int);
@@ -1254,13 +1107,40 @@ cudaError_t coarse_gmres(const Geom& g, const CoarseSolveArgs& ca, const R* b, R
                          int* iters, int* iters_acc, int* status, cudaStream_t st, const CoarsePlan* sized) {
   if (ca.restart > MAXM || ca.restart < 1 || nrhs < 1) return cudaErrorInvalidValue;
   const int n2 = 2 * ca.n;
-  Choice ch = choose<R>(g, n2, ca.restart, nrhs);
+  Choice ch = choose<R>(g, n2, ca.restart, nrhs, ca.wide != 0);
   if (ch.NR == 0) return cudaErrorInvalidConfiguration;
   // a caller that sized `work` for a plan must get exactly that plan
   if (sized && (sized->NR != ch.NR || sized->G != ch.G || sized->per != ch.per ||
                 sized->local_in_smem != (ch.local ? 1 : 0) || sized->resident != (ch.resident ? 1 : 0) ||
                 sized->ring != (ch.ring ? 1 : 0)))
     return cudaErrorInvalidValue;
+  int dev = 0;
+  cudaGetDevice(&dev);
+  // Cooperative launches from different streams (several batches served at
+  // once) must not overlap: each sizes its grid for the whole GPU and spins
+  // on a grid barrier, so two of them sharing the SMs could wait on each
+  // other's blocks.  Outside stream capture every launch waits for the
+  // previous one of the process on this device.
+  auto ordered = [&](auto&& launch) -> cudaError_t {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    cudaError_t e = cudaStreamIsCapturing(st, &cap);
+    if (e != cudaSuccess) return e;
+    const bool order = cap == cudaStreamCaptureStatusNone && dev >= 0 && dev < MAXDEV;
+    std::unique_lock<std::mutex> order_lock(g_coop_mu, std::defer_lock);
+    if (order) {
+      order_lock.lock();
+      if (!g_coop_done[dev]) e = cudaEventCreateWithFlags(&g_coop_done[dev], cudaEventDisableTiming);
+      else e = cudaStreamWaitEvent(st, g_coop_done[dev], 0);
+      if (e != cudaSuccess) return e;
+    }
+    e = launch();
+    ++g_launches;
+    if (e == cudaSuccess && order) e = cudaEventRecord(g_coop_done[dev], st);
+    return e;
+  };
+  if constexpr (sizeof(R) == 4)
+    if (ch.wide.NR)
+      return ordered([&] { return cgmres_wide_launch(ch.wide, g, ca, b, x, nrhs, work, iters, iters_acc, status, st); });
   CGA<R> a;
   a.g = g;
   a.Dc = reinterpret_cast<const cpx<R>*>(ca.Dc);
@@ -1279,7 +1159,6 @@ cudaError_t coarse_gmres(const Geom& g, const CoarseSolveArgs& ca, const R* b, R
   a.local_in_smem = ch.local ? 1 : 0;
   a.resident = ch.resident ? 1 : 0;
   a.ring = ch.ring ? 1 : 0;
-  a.tc = ca.tc;
   const size_t NE = a.NE;
   const size_t vec = (size_t)NRMAX * NE * n2;
   unsigned char* w8 = reinterpret_cast<unsigned char*>(work);
@@ -1301,35 +1180,11 @@ cudaError_t coarse_gmres(const Geom& g, const CoarseSolveArgs& ca, const R* b, R
   if (e != cudaSuccess) return e;
   const void* fn = kernel_for<R>(ch.NR);
   {
-    int dev = 0;
-    cudaGetDevice(&dev);
     std::lock_guard<std::mutex> lock(g_cfg_mu);
     e = smem_attr_locked<R>(dev, ch.NR, ch.plan.bytes);
   }
   if (e != cudaSuccess) return e;
   void* args[] = {&a};
-  // Cooperative launches from different streams (several batches served at
-  // once) must not overlap: each sizes its grid for the whole GPU and spins
-  // on a grid barrier, so two of them sharing the SMs could wait on each
-  // other's blocks.  Outside stream capture every launch waits for the
-  // previous one of the process on this device.
-  int dev = 0;
-  cudaGetDevice(&dev);
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  e = cudaStreamIsCapturing(st, &cap);
-  if (e != cudaSuccess) return e;
-  const bool order = cap == cudaStreamCaptureStatusNone && dev >= 0 && dev < MAXDEV;
-  std::unique_lock<std::mutex> order_lock(g_coop_mu, std::defer_lock);
-  if (order) {
-    order_lock.lock();
-    if (!g_coop_done[dev]) {
-      e = cudaEventCreateWithFlags(&g_coop_done[dev], cudaEventDisableTiming);
-      if (e != cudaSuccess) return e;
-    } else {
-      e = cudaStreamWaitEvent(st, g_coop_done[dev], 0);
-      if (e != cudaSuccess) return e;
-    }
-  }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(ch.G);
   cfg.blockDim = dim3(TPB);
@@ -1340,10 +1195,7 @@ cudaError_t coarse_gmres(const Geom& g, const CoarseSolveArgs& ca, const R* b, R
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  e = cudaLaunchKernelExC(&cfg, fn, args);
-  ++g_launches;
-  if (e == cudaSuccess && order) e = cudaEventRecord(g_coop_done[dev], st);
-  return e;
+  return ordered([&] { return cudaLaunchKernelExC(&cfg, fn, args); });
 }
 
 // A captured graph that holds a cooperative coarse-GMRES launch joins the
