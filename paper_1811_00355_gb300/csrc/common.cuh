@@ -143,7 +143,12 @@ __device__ __forceinline__ void load_units(const R* __restrict__ f, int d, int V
 // widths in reals
 constexpr int SPINOR_NR = 24;   // 4 spins x 3 colours complex
 constexpr int LINK_NR = 12;     // two rows of an SU(3) matrix
-constexpr int GAUGE_NR = 48;    // 4 links per site
+constexpr int GAUGE_NR = 48;    // 4 links per site as two rows
+// Links in FP32 are kept as two rows: bytes bound their kernels.  In FP64 the
+// third row is kept too: rebuilding it takes 24 of the 144 FP64 instructions of
+// a hop, and the FP64 pipe (2 lanes a clock and SM) bounds every FP64 kernel.
+constexpr int LINK64_NR = 18;
+constexpr int GAUGE64_NR = 72;
 constexpr int CLOVER_NR = 72;   // two packed Hermitian 6x6 blocks
 
 template <class R>
@@ -181,6 +186,15 @@ __device__ __forceinline__ void complete_link(Link<R>& U) {
 
 template <class R>
 __device__ __forceinline__ void load_link(const R* __restrict__ g, int d, int Vb, int mu, Link<R>& U) {
+  if constexpr (sizeof(R) == 8) {
+    const size_t b = Layout<double, GAUGE64_NR>::base(d, Vb) + (size_t)(mu * 9) * Vb;
+#pragma unroll
+    for (int u = 0; u < 9; ++u) {
+      const double2 t = __ldg(reinterpret_cast<const double2*>(g) + b + (size_t)u * Vb);
+      U.m[u / 3][u % 3] = mk(t.x, t.y);
+    }
+    return;
+  }
   using LY = Layout<R, GAUGE_NR>;
   constexpr int NUL = LINK_NR / LY::PER;   // units per link
   R v[LINK_NR];
@@ -246,6 +260,23 @@ __device__ __forceinline__ void project(const Spinor<R>& p, cpx<R> h[2][3]) {
       if (SIGN < 0) { h[0][a] = s0 - s2; h[1][a] = s1 - s3; }
       else          { h[0][a] = s0 + s2; h[1][a] = s1 + s3; }
     }
+  }
+}
+
+// y times -1 where the bit (31) of e is set: the sign of a hop across the time
+// boundary, without an instruction of the FP64 pipe
+__device__ __forceinline__ void flip_sign(cpx<float> (&y)[2][3], uint32_t e) {
+  const float s = (e & 0x80000000u) ? -1.f : 1.f;
+#pragma unroll
+  for (int k = 0; k < 6; ++k) y[k / 3][k % 3] = s * y[k / 3][k % 3];
+}
+__device__ __forceinline__ void flip_sign(cpx<double> (&y)[2][3], uint32_t e) {
+  const int bit = (int)(e & 0x80000000u);
+#pragma unroll
+  for (int k = 0; k < 6; ++k) {
+    cpx<double>& v = y[k / 3][k % 3];
+    v.re = __hiloint2double(__double2hiint(v.re) ^ bit, __double2loint(v.re));
+    v.im = __hiloint2double(__double2hiint(v.im) ^ bit, __double2loint(v.im));
   }
 }
 
@@ -361,24 +392,24 @@ __device__ __forceinline__ void hop_dir(const Geom& g, const R* __restrict__ x,
   {  // forward: (1 - g_mu) U_mu(x) x(x+mu)
     uint32_t e = __ldg(g.nbr + (size_t)(2 * MU) * g.V + d);
     int n = (int)(e & ~NEG_BIT);
-    R sc = (e & NEG_BIT) ? R(-1) : R(1);
     load_spinor<R>(x, n, g.Vb, nb);
     project<MU, -1>(nb, h);
     Link<R> U;
     load_link<R>(gauge, d, g.Vb, MU, U);
     su3_mul(U, h, y);
-    accumulate<MU, -1>(acc, y, sc);
+    if (MU == 3) flip_sign(y, e);      // (only hops in t change sign)
+    accumulate<MU, -1>(acc, y, R(1));
   }
   {  // backward: (1 + g_mu) U_mu(x-mu)^H x(x-mu)
     uint32_t e = __ldg(g.nbr + (size_t)(2 * MU + 1) * g.V + d);
     int n = (int)(e & ~NEG_BIT);
-    R sc = (e & NEG_BIT) ? R(-1) : R(1);
     load_spinor<R>(x, n, g.Vb, nb);
     project<MU, +1>(nb, h);
     Link<R> U;
     load_link<R>(gauge, n, g.Vb, MU, U);
     su3_mul_dag(U, h, y);
-    accumulate<MU, +1>(acc, y, sc);
+    if (MU == 3) flip_sign(y, e);
+    accumulate<MU, +1>(acc, y, R(1));
   }
 }
 

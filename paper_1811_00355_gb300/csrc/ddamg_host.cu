@@ -80,7 +80,6 @@ struct ddamg_ctx {
   int* d_cpos = nullptr;
 
   // gauge and clover
-  double* d_gauge_lex = nullptr;
   double* g64 = nullptr;
   float* g32 = nullptr;
   double *A64 = nullptr, *Ai64 = nullptr;
@@ -595,6 +594,18 @@ ddamg_status import_fields(ddamg_ctx* h, const double* src, int on_device, int n
     lex = h->lexbuf;
   }
   CK(pack_spinor<R>(h->g, lex, dst, nf, h->st));
+  return DDAMG_OK;
+}
+// lexicographic FP64 links (72 doubles a site: staged like three fields when
+// they come from the host)
+ddamg_status import_links(ddamg_ctx* h, const double* src, int on_device) {
+  const double* lex = src;
+  if (!on_device) {
+    TRY(need_lexbuf(h, 3));
+    CK(cudaMemcpyAsync(h->lexbuf, src, 3 * h->V24 * sizeof(double), cudaMemcpyHostToDevice, h->st));
+    lex = h->lexbuf;
+  }
+  CK(import_gauge(h->g, lex, h->g64, h->g32, h->d_dev, h->st));
   return DDAMG_OK;
 }
 template <class R>
@@ -1359,7 +1370,7 @@ ddamg_status half_operators(ddamg_ctx* h, int k) {
 // half copies already in use are refreshed at once (captured graphs read
 // them in place)
 ddamg_status rebuild_clover(ddamg_ctx* h, double m0, double csw) {
-  CK(build_clover(h->g, h->d_gauge_lex, m0, csw, h->A64, h->Ai64, h->A32, h->Ai32, h->st));
+  CK(build_clover(h->g, h->g64, m0, csw, h->A64, h->Ai64, h->A32, h->Ai32, h->st));
   ++h->op_gen;
   for (int k = 0; k < 2; ++k)
     if (h->gH[k]) TRY(half_operators(h, k));
@@ -2504,8 +2515,7 @@ ddamg_status ddamg_create(const ddamg_params* p, const double* gauge, int gauge_
     TRY(build_tables(h));
     h->V24 = (size_t)h->g.V * 24;
     const size_t V = h->g.V;
-    TRY(dalloc_t(h, &h->d_gauge_lex, V * 72));
-    TRY(dalloc_t(h, &h->g64, V * 48));
+    TRY(dalloc_t(h, &h->g64, V * 72));
     TRY(dalloc_t(h, &h->g32, V * 48));
     TRY(dalloc_t(h, &h->A64, V * 72));
     TRY(dalloc_t(h, &h->Ai64, V * 72));
@@ -2525,9 +2535,7 @@ ddamg_status ddamg_create(const ddamg_params* p, const double* gauge, int gauge_
     TRY(dalloc_t(h, &h->lam64, (size_t)p->n_v * h->V24));
     CK(cudaMemsetAsync(h->d_status, 0, sizeof(int), h->st));
     CK(cudaMemsetAsync(h->d_dev, 0, sizeof(unsigned long long), h->st));
-    CK(cudaMemcpyAsync(h->d_gauge_lex, gauge, V * 72 * sizeof(double),
-                       gauge_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, h->st));
-    CK(import_gauge(h->g, h->d_gauge_lex, h->g64, h->g32, h->d_dev, h->st));
+    TRY(import_links(h, gauge, gauge_on_device));
     unsigned long long bits = 0;
     CK(cudaMemcpyAsync(&bits, h->d_dev, sizeof bits, cudaMemcpyDeviceToHost, h->st));
     CK(cudaStreamSynchronize(h->st));
@@ -2550,11 +2558,8 @@ ddamg_status ddamg_create(const ddamg_params* p, const double* gauge, int gauge_
 
 ddamg_status ddamg_set_gauge(ddamg_handle h, const double* gauge, int on_device) {
   if (!h || !gauge) return DDAMG_EINVAL;
-  const size_t V = h->g.V;
-  CK(cudaMemcpyAsync(h->d_gauge_lex, gauge, V * 72 * sizeof(double),
-                     on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, h->st));
   CK(cudaMemsetAsync(h->d_dev, 0, sizeof(unsigned long long), h->st));
-  CK(import_gauge(h->g, h->d_gauge_lex, h->g64, h->g32, h->d_dev, h->st));
+  TRY(import_links(h, gauge, on_device));
   unsigned long long bits = 0;
   CK(cudaMemcpyAsync(&bits, h->d_dev, sizeof bits, cudaMemcpyDeviceToHost, h->st));
   CK(cudaStreamSynchronize(h->st));

@@ -75,13 +75,14 @@ template <class RD, class RS>
 cudaError_t convert_spinor(const Geom& g, const RS* src, RD* dst, int nf, cudaStream_t st);
 
 // ---- gauge and clover -------------------------------------------------------
-// compress lexicographic FP64 links into the two-row device layouts; the
+// lexicographic FP64 links into the device layouts (three rows in FP64, the
+// third rebuilt; two in FP32); the
 // largest deviation from SU(3) (|U U^H - 1|, |det U - 1|) is max-reduced into
 // *dev_dev (as ordered bits of a non-negative double)
 cudaError_t import_gauge(const Geom& g, const double* lex, double* g64, float* g32,
                          unsigned long long* dev_dev, cudaStream_t st);
 // A = (4 + m0) + C and A^-1, packed, in FP64 and FP32 device layouts
-cudaError_t build_clover(const Geom& g, const double* lex_gauge, double m0, double csw,
+cudaError_t build_clover(const Geom& g, const double* g64, double m0, double csw,
                          double* A64, double* Ai64, float* A32, float* Ai32, cudaStream_t st);
 // export packed blocks to [lex site][2][36] doubles
 cudaError_t export_clover(const Geom& g, const double* dev, double* lex, cudaStream_t st);

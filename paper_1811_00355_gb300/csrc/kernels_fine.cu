@@ -170,6 +170,17 @@ __device__ __forceinline__ M3 ld_lex_link(const double* __restrict__ lex, int si
     for (int j = 0; j < 3; ++j) U.a[i][j] = mk(p[(i * 3 + j) * 2], p[(i * 3 + j) * 2 + 1]);
   return U;
 }
+// link mu of device site d from the FP64 device links
+__device__ __forceinline__ M3 ld_dev_link(const double* __restrict__ g64, int Vb, int d, int mu) {
+  Link<double> U;
+  load_link<double>(g64, d, Vb, mu, U);
+  M3 r;
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int j = 0; j < 3; ++j) r.a[i][j] = U.m[i][j];
+  return r;
+}
 __device__ __forceinline__ M3 mul(const M3& A, const M3& B) {
   M3 C;
 #pragma unroll
@@ -198,17 +209,6 @@ __device__ __forceinline__ M3 add(const M3& A, const M3& B) {
 #pragma unroll
     for (int j = 0; j < 3; ++j) C.a[i][j] = A.a[i][j] + B.a[i][j];
   return C;
-}
-
-__device__ __forceinline__ int lex_shift(int site, int mu, int step, const int* L) {
-  int c[4];
-  int r = site;
-  c[0] = r % L[0]; r /= L[0];
-  c[1] = r % L[1]; r /= L[1];
-  c[2] = r % L[2]; r /= L[2];
-  c[3] = r;
-  c[mu] = (c[mu] + step + L[mu]) % L[mu];
-  return c[0] + L[0] * (c[1] + L[1] * (c[2] + L[2] * c[3]));
 }
 
 // B_mu of g_mu = [[0, B], [B^H, 0]]
@@ -279,14 +279,15 @@ __device__ __forceinline__ void pack6(const c64 (&m)[6][6], double* P) {
 }
 
 // ---------------------------------------------------------------------------
-// gauge import: two rows of each link in both precisions + SU(3) check
+// gauge import: two rows of each link in FP32, with the third row rebuilt from
+// them in FP64, + SU(3) check
 // ---------------------------------------------------------------------------
 __global__ void k_import_gauge(Geom g, const double* __restrict__ lex, double* __restrict__ g64,
                                float* __restrict__ g32, unsigned long long* dev_dev) {
   int d = blockIdx.x * blockDim.x + threadIdx.x;
   if (d >= g.V) return;
   int x = g.lex_of_dev[d];
-  double v64[GAUGE_NR];
+  double v64[GAUGE64_NR];
   double worst = 0.0;
   for (int mu = 0; mu < 4; ++mu) {
     M3 U = ld_lex_link(lex, x, mu);
@@ -302,14 +303,17 @@ __global__ void k_import_gauge(Geom g, const double* __restrict__ lex, double* _
               U.a[0][2] * (U.a[1][0] * U.a[2][1] - U.a[1][1] * U.a[2][0]);
     worst = fmax(worst, sqrt(norm2(det - mk(1.0, 0.0))));
     if (!(worst == worst)) worst = 1e300;   // NaN
-    for (int k = 0; k < 6; ++k) {
-      v64[mu * 12 + 2 * k] = U.a[k / 3][k % 3].re;
-      v64[mu * 12 + 2 * k + 1] = U.a[k / 3][k % 3].im;
+    Link<double> T;
+    for (int k = 0; k < 6; ++k) T.m[k / 3][k % 3] = U.a[k / 3][k % 3];
+    complete_link(T);
+    for (int k = 0; k < 9; ++k) {
+      v64[mu * LINK64_NR + 2 * k] = T.m[k / 3][k % 3].re;
+      v64[mu * LINK64_NR + 2 * k + 1] = T.m[k / 3][k % 3].im;
     }
   }
-  store_site<double, GAUGE_NR>(g64, d, g.Vb, v64);
+  store_site<double, GAUGE64_NR>(g64, d, g.Vb, v64);
   float v32[GAUGE_NR];
-  for (int k = 0; k < GAUGE_NR; ++k) v32[k] = (float)v64[k];
+  for (int k = 0; k < GAUGE_NR; ++k) v32[k] = (float)v64[(k / LINK_NR) * LINK64_NR + k % LINK_NR];
   store_site<float, GAUGE_NR>(g32, d, g.Vb, v32);
   atomicMax(dev_dev, (unsigned long long)__double_as_longlong(worst));
 }
@@ -318,11 +322,14 @@ __global__ void k_import_gauge(Geom g, const double* __restrict__ lex, double* _
 // clover term C = -(csw/16) sum_{mu<nu} g_mu g_nu (x) (Q_munu - Q_munu^H),
 // chiral blocks: g_mu g_nu = diag(B_mu B_nu^H, B_mu^H B_nu)
 // ---------------------------------------------------------------------------
-__global__ void k_build_clover(Geom g, const double* __restrict__ lex, double m0, double csw,
+__global__ void k_build_clover(Geom g, const double* __restrict__ g64, double m0, double csw,
                                double* A64, double* Ai64, float* A32, float* Ai32) {
   int d = blockIdx.x * blockDim.x + threadIdx.x;
   if (d >= g.V) return;
-  int x = g.lex_of_dev[d];
+  auto step = [&](int at, int mu, int back) {
+    return (int)(__ldg(g.nbr + (size_t)(2 * mu + back) * g.V + at) & ~NEG_BIT);
+  };
+  auto link = [&](int at, int mu) { return ld_dev_link(g64, g.Vb, at, mu); };
   c64 blk[2][6][6];
   for (int s = 0; s < 2; ++s)
     for (int i = 0; i < 6; ++i)
@@ -330,20 +337,15 @@ __global__ void k_build_clover(Geom g, const double* __restrict__ lex, double m0
   const double coef = -csw / 16.0;
   for (int mu = 0; mu < 4; ++mu) {
     for (int nu = mu + 1; nu < 4; ++nu) {
-      int xpm = lex_shift(x, mu, 1, g.L), xpn = lex_shift(x, nu, 1, g.L);
-      int xmm = lex_shift(x, mu, -1, g.L), xmn = lex_shift(x, nu, -1, g.L);
-      int xmm_pn = lex_shift(xmm, nu, 1, g.L), xmm_mn = lex_shift(xmm, nu, -1, g.L);
-      int xmn_pm = lex_shift(xmn, mu, 1, g.L);
-      M3 Umx = ld_lex_link(lex, x, mu), Unx = ld_lex_link(lex, x, nu);
-      M3 l1 = mul(mul(Umx, ld_lex_link(lex, xpm, nu)), mul(dag(ld_lex_link(lex, xpn, mu)), dag(Unx)));
-      M3 Umm = ld_lex_link(lex, xmm, mu);
-      M3 l2 = mul(mul(Unx, dag(ld_lex_link(lex, xmm_pn, mu))),
-                  mul(dag(ld_lex_link(lex, xmm, nu)), Umm));
-      M3 l3 = mul(mul(dag(Umm), dag(ld_lex_link(lex, xmm_mn, nu))),
-                  mul(ld_lex_link(lex, xmm_mn, mu), ld_lex_link(lex, xmn, nu)));
-      M3 Unm = ld_lex_link(lex, xmn, nu);
-      M3 l4 = mul(mul(dag(Unm), ld_lex_link(lex, xmn, mu)),
-                  mul(ld_lex_link(lex, xmn_pm, nu), dag(Umx)));
+      const int xpm = step(d, mu, 0), xpn = step(d, nu, 0), xmm = step(d, mu, 1), xmn = step(d, nu, 1);
+      const int xmm_pn = step(xmm, nu, 0), xmm_mn = step(xmm, nu, 1), xmn_pm = step(xmn, mu, 0);
+      M3 Umx = link(d, mu), Unx = link(d, nu);
+      M3 l1 = mul(mul(Umx, link(xpm, nu)), mul(dag(link(xpn, mu)), dag(Unx)));
+      M3 Umm = link(xmm, mu);
+      M3 l2 = mul(mul(Unx, dag(link(xmm_pn, mu))), mul(dag(link(xmm, nu)), Umm));
+      M3 l3 = mul(mul(dag(Umm), dag(link(xmm_mn, nu))), mul(link(xmm_mn, mu), link(xmn, nu)));
+      M3 Unm = link(xmn, nu);
+      M3 l4 = mul(mul(dag(Unm), link(xmn, mu)), mul(link(xmn_pm, nu), dag(Umx)));
       M3 Q = add(add(l1, l2), add(l3, l4));
       M3 Qd = dag(Q);
       for (int s = 0; s < 2; ++s) {
@@ -395,14 +397,18 @@ __global__ void k_export_clover(Geom g, const double* __restrict__ dev, double* 
 // ---------------------------------------------------------------------------
 // Wilson-clover stencil, one thread per site
 // ---------------------------------------------------------------------------
+// (CTAs of one range of sites for all right-hand sides follow one another: the
+// links and clover blocks, five of the seven or eight fields a right-hand side
+// reads, come from DRAM once and from L2 for the others)
 template <class R, int MODE>
 __global__ void __launch_bounds__(TPB) k_dslash(Geom g, const R* __restrict__ x,
                                                 const R* __restrict__ b, R* __restrict__ y,
                                                 const R* __restrict__ gauge,
-                                                const R* __restrict__ clover) {
-  int d = blockIdx.x * blockDim.x + threadIdx.x;
+                                                const R* __restrict__ clover, int nrhs) {
+  const int rhs = blockIdx.x % nrhs;
+  int d = (blockIdx.x / nrhs) * blockDim.x + threadIdx.x;
   if (d >= g.V) return;
-  size_t off = (size_t)blockIdx.y * g.V * SPINOR_NR;
+  size_t off = (size_t)rhs * g.V * SPINOR_NR;
   x += off;
   y += off;
   Spinor<R> out;
@@ -786,9 +792,9 @@ cudaError_t import_gauge(const Geom& g, const double* lex, double* g64, float* g
   return cudaGetLastError();
 }
 
-cudaError_t build_clover(const Geom& g, const double* lex_gauge, double m0, double csw,
+cudaError_t build_clover(const Geom& g, const double* g64, double m0, double csw,
                          double* A64, double* Ai64, float* A32, float* Ai32, cudaStream_t st) {
-  k_build_clover<<<nblk(g.V, 64), 64, 0, st>>>(g, lex_gauge, m0, csw, A64, Ai64, A32, Ai32);
+  k_build_clover<<<nblk(g.V, 64), 64, 0, st>>>(g, g64, m0, csw, A64, Ai64, A32, Ai32);
   ++g_launches;
   return cudaGetLastError();
 }
@@ -802,13 +808,17 @@ cudaError_t export_clover(const Geom& g, const double* dev, double* lex, cudaStr
 template <class R>
 cudaError_t dslash(const Geom& g, int mode, const R* x, const R* b, R* y, const R* gauge,
                    const R* clover, int nrhs, cudaStream_t st) {
-  dim3 grid(nblk(g.V, TPB), nrhs);
+  // small lattices: single-warp CTAs reach all SMs (an 8^4 lattice has 32 CTAs
+  // of 128 threads; the FP64 D is bound by each SM's FP64 pipe)
+  int threads = TPB;
+  while (threads > 32 && (size_t)nblk(g.V, threads) * nrhs < 1216) threads /= 2;
+  const unsigned grid = nblk(g.V, threads) * (unsigned)nrhs;
   if (mode == DSLASH_D)
-    k_dslash<R, DSLASH_D><<<grid, TPB, 0, st>>>(g, x, b, y, gauge, clover);
+    k_dslash<R, DSLASH_D><<<grid, threads, 0, st>>>(g, x, b, y, gauge, clover, nrhs);
   else if (mode == DSLASH_RES)
-    k_dslash<R, DSLASH_RES><<<grid, TPB, 0, st>>>(g, x, b, y, gauge, clover);
+    k_dslash<R, DSLASH_RES><<<grid, threads, 0, st>>>(g, x, b, y, gauge, clover, nrhs);
   else
-    k_dslash<R, DSLASH_CLOVER><<<grid, TPB, 0, st>>>(g, x, b, y, gauge, clover);
+    k_dslash<R, DSLASH_CLOVER><<<grid, threads, 0, st>>>(g, x, b, y, gauge, clover, nrhs);
   ++g_launches;
   return cudaGetLastError();
 }

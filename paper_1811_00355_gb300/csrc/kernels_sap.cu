@@ -342,10 +342,12 @@ __global__ void __launch_bounds__(512) k_sap_sweep(Geom g, int colour, int mr_it
 
   // stage the block's links (contiguous in the block-major layout)
   {
-    const T16<R>* src = reinterpret_cast<const T16<R>*>(gauge) + (size_t)B * LYG::NU * Vb;
+    // (two rows of each link; FP64 links have a third one in between)
+    constexpr int NUL = LYG::NU / 4, NULG = sizeof(R) == 8 ? LINK64_NR / 2 : NUL;
+    const T16<R>* src = reinterpret_cast<const T16<R>*>(gauge) + (size_t)B * 4 * NULG * Vb;
     for (int i = threadIdx.x; i < LYG::NU * Vb; i += blockDim.x) {
       int u = i / Vb, q = i - u * Vb;
-      sl[u * Vbp + q] = __ldg(src + i);
+      sl[u * Vbp + q] = __ldg(src + (size_t)((u / NUL) * NULG + u % NUL) * Vb + q);
     }
   }
 
