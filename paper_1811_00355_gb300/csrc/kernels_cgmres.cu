@@ -32,8 +32,10 @@ namespace {
 
 constexpr int TPB = 512;
 // partial-sum groups of mrhs_matvec (the plan's mvp buffer): more column
-// chunks for few right-hand sides, fewer where the buffer grows with NR
-__host__ __device__ constexpr int mvp_groups(int NR) { return NR >= 8 ? 9 : 18; }
+// chunks for few right-hand sides, fewer where the buffer grows with NR.  (One
+// right-hand side in FP32: three chunks of each of eight blocks keep 480 of the
+// 512 threads busy with n_v 20, two 320)
+__host__ __device__ constexpr int mvp_groups(int NR, size_t rs) { return NR >= 8 ? 9 : NR == 1 && rs == 4 ? 24 : 18; }
 // row stride (complex entries) of the staged vectors sv[r][d][.]: one more
 // than n2, so that rows of different directions and right-hand sides read
 // at the same column fall on different shared-memory banks
@@ -83,15 +85,15 @@ __host__ __device__ inline Plan make_plan(int NR, int L, int n2, int m, int rs, 
     lb = g;
   }
   p.sv = put((size_t)NR * 9 * sv_stride(n2) * c);
-  p.mvp = put((size_t)mvp_groups(NR) * NR * n2 * c);
+  p.mvp = put((size_t)mvp_groups(NR, rs) * NR * n2 * c);
   p.tmp = put((size_t)NR * n2 * c);
-  p.hc = put((size_t)NR * 2 * (m + 1) * 8);
-  p.h2 = put((size_t)NR * 2 * (m + 1) * 8);
-  p.Rf = put((size_t)NR * m * (m + 1) * 8);
-  p.cs = put((size_t)NR * m * 8);
-  p.sn = put((size_t)NR * 2 * m * 8);
-  p.gv = put((size_t)NR * 2 * (m + 1) * 8);
-  p.yv = put((size_t)NR * 2 * m * 8);
+  p.hc = put((size_t)NR * 2 * (m + 1) * rs);
+  p.h2 = put((size_t)NR * 2 * (m + 1) * rs);
+  p.Rf = put((size_t)NR * m * (m + 1) * rs);
+  p.cs = put((size_t)NR * m * rs);
+  p.sn = put((size_t)NR * 2 * m * rs);
+  p.gv = put((size_t)NR * 2 * (m + 1) * rs);
+  p.yv = put((size_t)NR * 2 * m * rs);
   p.beta = put((size_t)NR * 8);
   p.bnorm = put((size_t)NR * 8);
   p.hn = put((size_t)NR * 8);
@@ -132,7 +134,7 @@ struct CGA {
   cpx<R>* xg;        // [NR][NE][n2]
   unsigned char* lglob;   // per-CTA local arrays when they do not fit in smem
   size_t lstride;         // bytes per CTA in lglob
-  double* part;      // [(MAXM + 2) * NR][G][2]
+  cpx<R>* part;      // [(MAXM + 2) * NR][G]
   unsigned* bar;
   int* iters;
   int* iters_acc;
@@ -169,7 +171,7 @@ __device__ __forceinline__ void mrhs_matvec(const cpx<R>* __restrict__ M, const 
   const int ND = d1 - d0;
   // column chunks: enough units for every thread, at most mvp_groups(NR) groups
   int CC = (int)blockDim.x / (ND * NP * RS);
-  if (CC * ND > mvp_groups(NR)) CC = mvp_groups(NR) / ND;
+  if (CC * ND > mvp_groups(NR, sizeof(R))) CC = mvp_groups(NR, sizeof(R)) / ND;
   if (CC < 1) CC = 1;
   if (CC > n2) CC = n2;
   const int CW = (n2 + CC - 1) / CC;
@@ -355,7 +357,7 @@ __global__ void __launch_bounds__(TPB) k_cgmres(CGA<R> a) {
       // this thread's unit: row pair j, right-hand-side slice rs, column chunk cc
       const int NP = n2 / RPU;
       int CC = TPB / (NP * RS);
-      if (CC > mvp_groups(NR)) CC = mvp_groups(NR);
+      if (CC > mvp_groups(NR, sizeof(R))) CC = mvp_groups(NR, sizeof(R));
       if (CC > n2) CC = n2;
       if (CC < 1) CC = 1;
       const int CW = (n2 + CC - 1) / CC;
@@ -510,8 +512,7 @@ __global__ void __launch_bounds__(TPB) k_cgmres(CGA<R> a) {
       re = wsum(re);
       im = wsum(im);
       if (lane == 0) {
-        a.part[((size_t)pr * G + blockIdx.x) * 2] = (double)re;
-        a.part[((size_t)pr * G + blockIdx.x) * 2 + 1] = (double)im;
+        a.part[(size_t)pr * G + blockIdx.x] = mk(re, im);
       }
     }
   };
@@ -521,8 +522,9 @@ __global__ void __launch_bounds__(TPB) k_cgmres(CGA<R> a) {
     for (int pr = wid; pr < pairs; pr += NW) {
       A re = 0, im = 0;
       for (int c = lane; c < G; c += 32) {
-        re += (A)__ldcg(a.part + ((size_t)pr * G + c) * 2);
-        im += (A)__ldcg(a.part + ((size_t)pr * G + c) * 2 + 1);
+        const cpx<R> z = ldc(a.part + (size_t)pr * G + c);
+        re += z.re;
+        im += z.im;
       }
       re = wsum(re);
       im = wsum(im);
@@ -541,23 +543,34 @@ __global__ void __launch_bounds__(TPB) k_cgmres(CGA<R> a) {
 
   // gather(kcount, false, hc, dstride) and gather_norm_slot(kcount, hn) in
   // one pass: one round of L2 loads instead of two
+  // (a warp's loads for four pairs go out together: an L2 round trip is most of
+  // the time, and 30 basis vectors are two pairs a warp)
   auto gather_dots_norm = [&](int kcount, A* dst, int dstride, A* hn) {
     const int pairs = (kcount + 1) * NR;
-    for (int pr = wid; pr < pairs; pr += NW) {
-      A re = 0, im = 0;
-      for (int c = lane; c < G; c += 32) {
-        re += (A)__ldcg(a.part + ((size_t)pr * G + c) * 2);
-        im += (A)__ldcg(a.part + ((size_t)pr * G + c) * 2 + 1);
-      }
-      re = wsum(re);
-      im = wsum(im);
-      if (lane == 0) {
-        const int j = pr / NR, r = pr - j * NR;
-        if (j < kcount) {
-          dst[(size_t)r * dstride + 2 * j] = re;
-          dst[(size_t)r * dstride + 2 * j + 1] = im;
-        } else {
-          hn[r] = re;                  // squared norm (real)
+    for (int p0 = wid; p0 < pairs; p0 += 4 * NW) {
+      A re[4] = {}, im[4] = {};
+      for (int c = lane; c < G; c += 32)
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if (p0 + q * NW < pairs) {
+            const cpx<R> z = ldc(a.part + (size_t)(p0 + q * NW) * G + c);
+            re[q] += z.re;
+            im[q] += z.im;
+          }
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int pr = p0 + q * NW;
+        if (pr >= pairs) break;
+        re[q] = wsum(re[q]);
+        im[q] = wsum(im[q]);
+        if (lane == 0) {
+          const int j = pr / NR, r = pr - j * NR;
+          if (j < kcount) {
+            dst[(size_t)r * dstride + 2 * j] = re[q];
+            dst[(size_t)r * dstride + 2 * j + 1] = im[q];
+          } else {
+            hn[r] = re[q];                  // squared norm (real)
+          }
         }
       }
     }
@@ -575,22 +588,10 @@ __global__ void __launch_bounds__(TPB) k_cgmres(CGA<R> a) {
       sq = wsum(sq);
       if (lane == 0) {
         const size_t pr = (size_t)kcount * NR + r;
-        a.part[(pr * G + blockIdx.x) * 2] = (double)sq;
-        a.part[(pr * G + blockIdx.x) * 2 + 1] = 0.0;
+        a.part[pr * G + blockIdx.x] = mk(sq, R(0));
       }
     }
   };
-  auto gather_norm_slot = [&](int kcount, A* dst) {
-    for (int r = wid; r < NR; r += NW) {
-      const size_t pr = (size_t)kcount * NR + r;
-      A sq = 0;
-      for (int c = lane; c < G; c += 32) sq += (A)__ldcg(a.part + (pr * G + c) * 2);
-      sq = wsum(sq);
-      if (lane == 0) dst[r] = sq;
-    }
-    __syncthreads();
-  };
-
   for (int r0 = 0; r0 < a.nrhs; r0 += NR) {
     const int nr = min(NR, a.nrhs - r0);
     const cpx<R>* bb = a.b + (size_t)r0 * a.g.nb * n2;
@@ -669,19 +670,25 @@ __global__ void __launch_bounds__(TPB) k_cgmres(CGA<R> a) {
         // thread), new residual estimate, scale 1/h of V_{k+1}, convergence
         auto givens = [&](int r) {
           const A hn = sqrt(hnv[r]);
-          A* col = hc + (size_t)r * 2 * (m + 1);   // this column of the Hessenberg matrix
-          col[2 * (k + 1)] = hn;
-          col[2 * (k + 1) + 1] = A(0);
-          A* csr = cs + (size_t)r * m;
-          A* snr = sn + (size_t)r * 2 * m;
+          const A* __restrict__ col = hc + (size_t)r * 2 * (m + 1);   // this column of the Hessenberg matrix
+          A* __restrict__ csr = cs + (size_t)r * m;
+          A* __restrict__ snr = sn + (size_t)r * 2 * m;
+          A* __restrict__ Rr = Rf + (size_t)r * 2 * TRI;
+          const int base = k * (k + 1) / 2;          // packed column k: entries 0..k
+          // the rotations so far: (ar, ai) runs down the column, its results
+          // go straight to the triangular factor, so the loads of the next
+          // steps need not wait for the chain
+          A ar = col[0], ai = col[1];
+#pragma unroll 4
           for (int j = 0; j < k; ++j) {
-            A c = csr[j], sr = snr[2 * j], si = snr[2 * j + 1];
-            A ar = col[2 * j], ai = col[2 * j + 1], br = col[2 * j + 2], bi = col[2 * j + 3];
-            A tr = c * ar + (sr * br - si * bi), ti = c * ai + (sr * bi + si * br);
-            A ur = -(sr * ar + si * ai) + c * br, ui = -(sr * ai - si * ar) + c * bi;
-            col[2 * j] = tr; col[2 * j + 1] = ti; col[2 * j + 2] = ur; col[2 * j + 3] = ui;
+            const A c = csr[j], sr = snr[2 * j], si = snr[2 * j + 1], br = col[2 * j + 2], bi = col[2 * j + 3];
+            Rr[2 * (base + j)] = c * ar + (sr * br - si * bi);
+            Rr[2 * (base + j) + 1] = c * ai + (sr * bi + si * br);
+            const A ur = c * br - (sr * ar + si * ai), ui = c * bi - (sr * ai - si * ar);
+            ar = ur;
+            ai = ui;
           }
-          A ar = col[2 * k], ai = col[2 * k + 1], br = col[2 * k + 2], bi = col[2 * k + 3];
+          const A br = hn, bi = A(0);
           A a1 = sqrt(ar * ar + ai * ai), a2 = sqrt(br * br + bi * bi);
           A c, sr, si, rr, ri;
           if (a2 == A(0)) { c = A(1); sr = A(0); si = A(0); rr = ar; ri = ai; }
@@ -695,10 +702,7 @@ __global__ void __launch_bounds__(TPB) k_cgmres(CGA<R> a) {
             rr = pr * rho; ri = pi * rho;
           }
           csr[k] = c; snr[2 * k] = sr; snr[2 * k + 1] = si;
-          col[2 * k] = rr; col[2 * k + 1] = ri;
-          A* Rr = Rf + (size_t)r * 2 * TRI;
-          const int base = k * (k + 1) / 2;          // packed column k: entries 0..k
-          for (int j = 0; j <= k; ++j) { Rr[2 * (base + j)] = col[2 * j]; Rr[2 * (base + j) + 1] = col[2 * j + 1]; }
+          Rr[2 * (base + k)] = rr; Rr[2 * (base + k) + 1] = ri;
           A* g = gv + (size_t)r * 2 * (m + 1);
           A gr = g[2 * k], gi = g[2 * k + 1];
           g[2 * (k + 1)] = -(sr * gr + si * gi);
@@ -1166,7 +1170,7 @@ cudaError_t coarse_gmres(const Geom& g, const CoarseSolveArgs& ca, const R* b, R
   a.to = a.wg + vec;
   a.xg = a.to + vec;
   size_t off = al16(3 * vec * sizeof(cpx<R>));
-  a.part = reinterpret_cast<double*>(w8 + off);
+  a.part = reinterpret_cast<cpx<R>*>(w8 + off);
   off += al16((size_t)(MAXM + 2) * NRMAX * NE * 2 * sizeof(double));
   a.bar = reinterpret_cast<unsigned*>(w8 + off);
   off += 256;

@@ -543,20 +543,22 @@ __global__ void __launch_bounds__(TPB, 1) k_cgmres_wide(WideArgs a) {
         // thread), new residual estimate, scale 1/h of V_{k+1}, convergence
         auto givens = [&](int r) {
           const float hn = sqrtf(hnv[r]);
-          float* col = hc + (size_t)r * 2 * (m + 1);   // this column of the Hessenberg matrix
-          col[2 * (k + 1)] = hn;
-          col[2 * (k + 1) + 1] = 0.f;
-          float* csr = cs + (size_t)r * m;
-          float* snr = sn + (size_t)r * 2 * m;
+          const float* __restrict__ col = hc + (size_t)r * 2 * (m + 1);   // this column of the Hessenberg matrix
+          float* __restrict__ csr = cs + (size_t)r * m;
+          float* __restrict__ snr = sn + (size_t)r * 2 * m;
+          float* __restrict__ Rr = Rf + (size_t)r * 2 * TRI;
+          const int base = k * (k + 1) / 2;          // packed column k: entries 0..k
+          float ar = col[0], ai = col[1];            // runs down the column through the rotations so far
+#pragma unroll 4
           for (int j = 0; j < k; ++j) {
-            const float c = csr[j], sr = snr[2 * j], si = snr[2 * j + 1];
-            const float ar = col[2 * j], ai = col[2 * j + 1], br = col[2 * j + 2], bi = col[2 * j + 3];
-            col[2 * j] = c * ar + (sr * br - si * bi);
-            col[2 * j + 1] = c * ai + (sr * bi + si * br);
-            col[2 * j + 2] = -(sr * ar + si * ai) + c * br;
-            col[2 * j + 3] = -(sr * ai - si * ar) + c * bi;
+            const float c = csr[j], sr = snr[2 * j], si = snr[2 * j + 1], br = col[2 * j + 2], bi = col[2 * j + 3];
+            Rr[2 * (base + j)] = c * ar + (sr * br - si * bi);
+            Rr[2 * (base + j) + 1] = c * ai + (sr * bi + si * br);
+            const float ur = c * br - (sr * ar + si * ai), ui = c * bi - (sr * ai - si * ar);
+            ar = ur;
+            ai = ui;
           }
-          const float ar = col[2 * k], ai = col[2 * k + 1], br = col[2 * k + 2], bi = col[2 * k + 3];
+          const float br = hn, bi = 0.f;
           const float a1 = sqrtf(ar * ar + ai * ai), a2 = sqrtf(br * br + bi * bi);
           float c, sr, si, rr, ri;
           if (a2 == 0.f) { c = 1.f; sr = 0.f; si = 0.f; rr = ar; ri = ai; }
@@ -569,10 +571,7 @@ __global__ void __launch_bounds__(TPB, 1) k_cgmres_wide(WideArgs a) {
             rr = pr * rho; ri = pi * rho;
           }
           csr[k] = c; snr[2 * k] = sr; snr[2 * k + 1] = si;
-          col[2 * k] = rr; col[2 * k + 1] = ri;
-          float* Rr = Rf + (size_t)r * 2 * TRI;
-          const int base = k * (k + 1) / 2;          // packed column k: entries 0..k
-          for (int j = 0; j <= k; ++j) { Rr[2 * (base + j)] = col[2 * j]; Rr[2 * (base + j) + 1] = col[2 * j + 1]; }
+          Rr[2 * (base + k)] = rr; Rr[2 * (base + k) + 1] = ri;
           float* g = gv + (size_t)r * 2 * (m + 1);
           const float gr = g[2 * k], gi = g[2 * k + 1];
           g[2 * (k + 1)] = -(sr * gr + si * gi);
