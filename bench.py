@@ -35,9 +35,11 @@ UNIT = "solves/s"
 WORKLOAD = dict(L=(16, 16, 16, 16), block=(4, 4, 4, 4), eps=0.25, seed=1, m0=-0.3, csw=1.2,
                 n_v=20, setup_iters=4, n_sap=4, mr_iters=4, coarse_tol=5e-2, tol=1e-10)
 # algorithmic (compulsory) bytes per site of one launch of each timed kernel,
-# FP32 storage with two-row links: SAP sweep reads b, x, 4 links, A, A^-1 and
-# writes x on its blocks (the coarse GMRES bytes are computed below).
-SAP_BYTES_PER_SITE = 4 * (24 + 24 + 24 + 48 + 72 + 72)
+# FP32 storage with two-row links: a SAP sweep reads 4 links and one clover
+# block (A on an even site, A^-1 on an odd one), reads and writes x, the even
+# sites' residual and the half spinors on the faces of its 4^4 blocks (the
+# coarse GMRES bytes are computed below).
+SAP_BYTES_PER_SITE = 4 * (48 + 72 + 24 + 24 + 12 + 12 + 24 + 24)
 L2_BYTES = 129 * 2 ** 20
 # DRAM bytes (read + write) per launch of each timed kernel class on this
 # workload, from an ncu capture of the kernel as it is now (a single-RHS
@@ -883,15 +885,16 @@ def stencils(P, torch, stream, pk, pk_kind):
             st = h.stats()
             h.enable_kernel_timing(False)
             us = 1e3 * st["dslash_ms"] / st["dslash_launches"]
-            # half storage: two site norms (FP32) besides the half values
-            byts = V * (D_REALS_PER_SITE * rs + (8 if rs == 2 else 0))
+            # half storage: two site norms (FP32) besides the half values;
+            # FP32 writes its output in FP64 (the exchange layout)
+            byts = V * (D_REALS_PER_SITE * rs + {2: 8, 4: 24 * 4, 8: 0}[rs])
             gbs = byts / (us * 1e-6) / 1e9
             out[name] = {"us": round(us, 2), "bytes_per_launch": byts, "GB/s": round(gbs, 1),
                          "frac": round(gbs / pk["hbm_gbs"], 4)}
         # one SAP application (4 cycles of the two colours from a zero start,
-        # single right-hand side): per sweep the sites of one colour read b,
-        # x (and their neighbours' x, from L2), links, A, A^-1 and write x
-        for name, prec, rs, extra in (("sap_sweep_f32", P.FP32, 4, 0), ("sap_sweep_bf16", P.BF16, 2, 12)):
+        # single right-hand side): per sweep the bytes of SAP_BYTES_PER_SITE,
+        # in half storage with half links and clover blocks
+        for name, prec, rs in (("sap_sweep_f32", P.FP32, 4), ("sap_sweep_bf16", P.BF16, 2)):
             for _ in range(2):
                 h.sap(x, prec)
             h.reset_stats()
@@ -901,7 +904,7 @@ def stencils(P, torch, stream, pk, pk_kind):
             st = h.stats()
             h.enable_kernel_timing(False)
             us = 1e3 * st["sap_ms"] / st["sap_launches"]
-            byts = (V // 2) * ((24 + 24 + 24 + 48 + 72 + 72) * rs + extra)
+            byts = (V // 2) * (SAP_BYTES_PER_SITE - (48 + 72) * (4 - rs))
             gbs = byts / (us * 1e-6) / 1e9
             out[name] = {"us": round(us, 2), "bytes_per_launch": byts, "GB/s": round(gbs, 1),
                          "frac": round(gbs / pk["hbm_gbs"], 4), "sweeps_timed": st["sap_launches"]}

@@ -384,15 +384,15 @@ constexpr uint32_t NEG_BIT = 0x80000000u;
 // global table, fields in global memory):
 //   acc += (1 - g_mu) U_mu(x) x(x+mu) + (1 + g_mu) U_mu(x-mu)^H x(x-mu)
 // ---------------------------------------------------------------------------
-template <int MU, class R>
-__device__ __forceinline__ void hop_dir(const Geom& g, const R* __restrict__ x,
-                                        const R* __restrict__ gauge, int d, Spinor<R>& acc) {
+// (spinor(n, s) loads the spinor of device site n)
+template <int MU, class R, class F>
+__device__ __forceinline__ void hop_dir(const Geom& g, F&& spinor, const R* __restrict__ gauge, int d, Spinor<R>& acc) {
   cpx<R> h[2][3], y[2][3];
   Spinor<R> nb;
   {  // forward: (1 - g_mu) U_mu(x) x(x+mu)
     uint32_t e = __ldg(g.nbr + (size_t)(2 * MU) * g.V + d);
     int n = (int)(e & ~NEG_BIT);
-    load_spinor<R>(x, n, g.Vb, nb);
+    spinor(n, nb);
     project<MU, -1>(nb, h);
     Link<R> U;
     load_link<R>(gauge, d, g.Vb, MU, U);
@@ -403,7 +403,7 @@ __device__ __forceinline__ void hop_dir(const Geom& g, const R* __restrict__ x,
   {  // backward: (1 + g_mu) U_mu(x-mu)^H x(x-mu)
     uint32_t e = __ldg(g.nbr + (size_t)(2 * MU + 1) * g.V + d);
     int n = (int)(e & ~NEG_BIT);
-    load_spinor<R>(x, n, g.Vb, nb);
+    spinor(n, nb);
     project<MU, +1>(nb, h);
     Link<R> U;
     load_link<R>(gauge, n, g.Vb, MU, U);

@@ -94,6 +94,12 @@ template <class R>
 cudaError_t dslash(const Geom& g, int mode, const R* x, const R* b, R* y, const R* gauge,
                    const R* clover, int nrhs, cudaStream_t st);
 
+// y = D x with y (and, lex_in, x; FP64 only) in the exchange layout; an x in
+// it must not overlap y
+template <class R>
+cudaError_t dslash_lex(const Geom& g, const R* x, bool lex_in, double* y, const R* gauge, const R* clover, int nrhs,
+                       cudaStream_t st);
+
 // ---- half-precision storage (S = __half or __nv_bfloat16; half.cuh) ------------
 // D in FP32 arithmetic with half links, clover blocks and spinors (each
 // spinor field with its FP32 site norms xn / bn / yn, V per field)

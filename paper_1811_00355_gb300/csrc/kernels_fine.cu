@@ -400,44 +400,96 @@ __global__ void k_export_clover(Geom g, const double* __restrict__ dev, double* 
 // (CTAs of one range of sites for all right-hand sides follow one another: the
 // links and clover blocks, five of the seven or eight fields a right-hand side
 // reads, come from DRAM once and from L2 for the others)
-template <class R, int MODE>
+//
+// LEX_IN (FP64), LEX_OUT: x, y in the exchange layout (lexicographic FP64)
+// instead of the device layout, for a single application on a caller's
+// fields.  FP64 is bound by its pipe, so the threads' strided 16-byte accesses
+// to x and y are free and the two conversion passes go; an FP32 y goes through
+// shared memory, whole sites at a time, and one pass goes (x is read eight
+// times and stays packed).  Call on 32^3 x 64 in FP32 and on 24^3 x 48 and 8^4
+// in FP64: see dslash_lex below.
+constexpr int LEX_IN = 1, LEX_OUT = 2;
+// spinor of device site d of x
+template <class R, int LEX>
+__device__ __forceinline__ void site_spinor(const Geom& g, const R* __restrict__ x, int d, Spinor<R>& s) {
+  if constexpr ((LEX & LEX_IN) != 0) {
+    const double* p = x + (size_t)__ldg(g.lex_of_dev + d) * SPINOR_NR;
+    const bool wide = (reinterpret_cast<uintptr_t>(x) & 15) == 0;
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {
+      const double2 v = lex_get(p + 2 * k, wide);
+      s.c[k] = mk(v.x, v.y);
+    }
+  } else {
+    load_spinor<R>(x, d, g.Vb, s);
+  }
+}
+template <class R, int MODE, int LEX = 0>
 __global__ void __launch_bounds__(TPB) k_dslash(Geom g, const R* __restrict__ x,
                                                 const R* __restrict__ b, R* __restrict__ y,
                                                 const R* __restrict__ gauge,
                                                 const R* __restrict__ clover, int nrhs) {
-  const int rhs = blockIdx.x % nrhs;
-  int d = (blockIdx.x / nrhs) * blockDim.x + threadIdx.x;
-  if (d >= g.V) return;
+  const int rhs = blockIdx.x % nrhs, first = (blockIdx.x / nrhs) * blockDim.x;
+  int d = first + threadIdx.x;
+  constexpr bool TILE_OUT = (LEX & LEX_OUT) != 0 && sizeof(R) == 4;
+  if (!TILE_OUT && d >= g.V) return;
   size_t off = (size_t)rhs * g.V * SPINOR_NR;
   x += off;
-  y += off;
   Spinor<R> out;
-  {
-    Spinor<R> xs;
-    load_spinor<R>(x, d, g.Vb, xs);
-    clover_mul<R>(clover, d, g.Vb, xs, out);
-  }
-  if (MODE != DSLASH_CLOVER) {
-    Spinor<R> acc;
+  if (d < g.V) {
+    {
+      Spinor<R> xs;
+      site_spinor<R, LEX>(g, x, d, xs);
+      clover_mul<R>(clover, d, g.Vb, xs, out);
+    }
+    if (MODE != DSLASH_CLOVER) {
+      Spinor<R> acc;
 #pragma unroll
-    for (int k = 0; k < 12; ++k) acc.c[k] = mk(R(0), R(0));
-    hop_dir<0>(g, x, gauge, d, acc);
-    hop_dir<1>(g, x, gauge, d, acc);
-    hop_dir<2>(g, x, gauge, d, acc);
-    hop_dir<3>(g, x, gauge, d, acc);
+      for (int k = 0; k < 12; ++k) acc.c[k] = mk(R(0), R(0));
+      auto spinor = [&](int n, Spinor<R>& s) { site_spinor<R, LEX>(g, x, n, s); };
+      hop_dir<0, R>(g, spinor, gauge, d, acc);
+      hop_dir<1, R>(g, spinor, gauge, d, acc);
+      hop_dir<2, R>(g, spinor, gauge, d, acc);
+      hop_dir<3, R>(g, spinor, gauge, d, acc);
 #pragma unroll
-    for (int k = 0; k < 12; ++k) {
-      out.c[k].re = fma_r(R(-0.5), acc.c[k].re, out.c[k].re);
-      out.c[k].im = fma_r(R(-0.5), acc.c[k].im, out.c[k].im);
+      for (int k = 0; k < 12; ++k) {
+        out.c[k].re = fma_r(R(-0.5), acc.c[k].re, out.c[k].re);
+        out.c[k].im = fma_r(R(-0.5), acc.c[k].im, out.c[k].im);
+      }
+    }
+    if (MODE == DSLASH_RES) {
+      Spinor<R> bs;
+      load_spinor<R>(b + off, d, g.Vb, bs);
+#pragma unroll
+      for (int k = 0; k < 12; ++k) out.c[k] = bs.c[k] - out.c[k];
     }
   }
-  if (MODE == DSLASH_RES) {
-    Spinor<R> bs;
-    load_spinor<R>(b + off, d, g.Vb, bs);
+  if constexpr ((LEX & LEX_OUT) == 0) {
+    store_spinor<R>(y + off, d, g.Vb, out);
+  } else {
+    double* lex = reinterpret_cast<double*>(y) + off;      // (y is the exchange buffer)
+    const bool wide = (reinterpret_cast<uintptr_t>(y) & 15) == 0;
+    if constexpr (sizeof(R) == 8) {
+      double* p = lex + (size_t)__ldg(g.lex_of_dev + d) * SPINOR_NR;
 #pragma unroll
-    for (int k = 0; k < 12; ++k) out.c[k] = bs.c[k] - out.c[k];
+      for (int k = 0; k < 12; ++k) lex_put(p + 2 * k, wide, make_double2(out.c[k].re, out.c[k].im));
+    } else {
+      __shared__ float2 tile[TPB * 13];          // 13: a site's components on different banks
+      __shared__ int at[TPB];
+      const int t = threadIdx.x, live = min((int)blockDim.x, g.V - first);
+      if (t < live) {
+        at[t] = g.lex_of_dev[d];
+#pragma unroll
+        for (int k = 0; k < 12; ++k) tile[t * 13 + k] = make_float2(out.c[k].re, out.c[k].im);
+      }
+      __syncthreads();
+      for (int it = t; it < 12 * live; it += blockDim.x) {
+        const int q = it / 12, k = it - 12 * q;
+        const float2 v = tile[q * 13 + k];
+        lex_put(lex + (size_t)at[q] * SPINOR_NR + 2 * k, wide, make_double2((double)v.x, (double)v.y));
+      }
+    }
   }
-  store_spinor<R>(y, d, g.Vb, out);
 }
 
 // ---------------------------------------------------------------------------
@@ -805,13 +857,17 @@ cudaError_t export_clover(const Geom& g, const double* dev, double* lex, cudaStr
   return cudaGetLastError();
 }
 
+// small lattices: single-warp CTAs reach all SMs (an 8^4 lattice has 32 CTAs
+// of 128 threads; the FP64 D is bound by each SM's FP64 pipe)
+static int dslash_threads(const Geom& g, int nrhs) {
+  int threads = TPB;
+  while (threads > 32 && (size_t)nblk(g.V, threads) * nrhs < 1216) threads /= 2;
+  return threads;
+}
 template <class R>
 cudaError_t dslash(const Geom& g, int mode, const R* x, const R* b, R* y, const R* gauge,
                    const R* clover, int nrhs, cudaStream_t st) {
-  // small lattices: single-warp CTAs reach all SMs (an 8^4 lattice has 32 CTAs
-  // of 128 threads; the FP64 D is bound by each SM's FP64 pipe)
-  int threads = TPB;
-  while (threads > 32 && (size_t)nblk(g.V, threads) * nrhs < 1216) threads /= 2;
+  const int threads = dslash_threads(g, nrhs);
   const unsigned grid = nblk(g.V, threads) * (unsigned)nrhs;
   if (mode == DSLASH_D)
     k_dslash<R, DSLASH_D><<<grid, threads, 0, st>>>(g, x, b, y, gauge, clover, nrhs);
@@ -822,6 +878,28 @@ cudaError_t dslash(const Geom& g, int mode, const R* x, const R* b, R* y, const 
   ++g_launches;
   return cudaGetLastError();
 }
+template <class R>
+cudaError_t dslash_lex(const Geom& g, const R* x, bool lex_in, double* y, const R* gauge, const R* clover, int nrhs,
+                       cudaStream_t st) {
+  const int threads = dslash_threads(g, nrhs);
+  const unsigned grid = nblk(g.V, threads) * (unsigned)nrhs;
+  R* out = reinterpret_cast<R*>(y);
+  if constexpr (sizeof(R) == 8) {
+    if (lex_in)
+      k_dslash<R, DSLASH_D, LEX_IN | LEX_OUT><<<grid, threads, 0, st>>>(g, x, nullptr, out, gauge, clover, nrhs);
+    else
+      k_dslash<R, DSLASH_D, LEX_OUT><<<grid, threads, 0, st>>>(g, x, nullptr, out, gauge, clover, nrhs);
+  } else {
+    if (lex_in) return cudaErrorInvalidValue;
+    k_dslash<R, DSLASH_D, LEX_OUT><<<grid, threads, 0, st>>>(g, x, nullptr, out, gauge, clover, nrhs);
+  }
+  ++g_launches;
+  return cudaGetLastError();
+}
+template cudaError_t dslash_lex<float>(const Geom&, const float*, bool, double*, const float*, const float*, int,
+                                       cudaStream_t);
+template cudaError_t dslash_lex<double>(const Geom&, const double*, bool, double*, const double*, const double*, int,
+                                        cudaStream_t);
 
 size_t reduce_scratch_len(int k) { return (size_t)k * RED_CTAS * 2; }
 

@@ -28,3 +28,26 @@ def test_D(L, block, nrhs):
         assert_close(s.apply_D(x, 1), ref, TOL32)
         assert_close(s.get_clover(), op.packed_clover().numpy(), TOL64)
     s.close()
+
+
+def test_fp64_D_in_place_and_unaligned():
+    """FP64 D on device buffers reads and writes them directly: also where the
+    output is the input (the neighbours are read first), overlaps it, or is
+    aligned to 8 bytes only; through the C interface, as the binding allocates
+    its own output."""
+    import ctypes as C
+    L, block = (8, 4, 4, 12), (4, 2, 2, 6)
+    x = syn.gaussian_spinors(2, L, 15)
+    ref = oracle_op(L, 0.3, 4, -0.2, 1.0).apply(t(x)).numpy()
+    s = make((L, block, 0.3, -0.2, 1.0, 1, 4), 1)
+    n = 2 * x.size
+    for prec, tol in ((0, TOL64), (1, TOL32)):
+        for shift, out_at in ((0, 0), (1, 1), (0, n), (1, n + 1), (0, n // 2), (1, n + 2)):
+            buf = torch.zeros(2 * n + 4, dtype=torch.float64, device="cuda")
+            buf[shift:shift + n] = torch.from_numpy(x.view(np.float64).reshape(-1)).cuda()
+            torch.cuda.synchronize()
+            at = lambda k: C.c_void_p(buf.data_ptr() + 8 * k)      # noqa: E731
+            assert s.lib.ddamg_apply_D(s.h, prec, 2, at(shift), at(out_at), 1) == 0
+            got = buf[out_at:out_at + n].cpu().numpy().view(np.complex128).reshape(x.shape)
+            assert_close(got, ref, tol, f"precision {prec} in {shift} out {out_at}")
+    s.close()
