@@ -1334,7 +1334,8 @@ ddamg_status sync_lam32(ddamg_ctx* h) {
   if (inner32(h)) {
     if (!h->lam32) TRY(dalloc_t(h, &h->lam32, (size_t)h->p.n_v * h->V24));
     // after ddamg_trim the FP32 copy is the only one (and current)
-    if (!h->lam64_gone) CK(convert_spinor<float, double>(h->g, h->lam64, h->lam32, h->p.n_v, h->st));
+    if (!h->lam64_gone && !h->lam32_fresh)
+      CK(convert_spinor<float, double>(h->g, h->lam64, h->lam32, h->p.n_v, h->st));
     h->lam32_fresh = true;
     const int k = lam_half_kind(h);
     if (k >= 0) {
@@ -1462,11 +1463,12 @@ ddamg_status coarse_iters_since(ddamg_ctx* h, int* its) {
 // them in FP32) on the FP32 copy, which the FP64 copy then takes
 ddamg_status ortho_inner(ddamg_ctx* h) {
   h->lam32_fresh = false;
+  if (inner32(h) && !h->lam32) TRY(dalloc_t(h, &h->lam32, (size_t)h->p.n_v * h->V24));
   if (!inner32(h) || !h->p.ortho_fp32) {
-    CK(orthonormalise(h->g, h->lam64, h->p.n_v, h->st));
+    CK(orthonormalise(h->g, h->lam64, inner32(h) ? h->lam32 : nullptr, h->p.n_v, h->st));
+    h->lam32_fresh = inner32(h);
     return DDAMG_OK;
   }
-  if (!h->lam32) TRY(dalloc_t(h, &h->lam32, (size_t)h->p.n_v * h->V24));
   CK(convert_spinor<float, double>(h->g, h->lam64, h->lam32, h->p.n_v, h->st));
   CK(orthonormalise(h->g, h->lam32, h->p.n_v, h->st));
   CK(convert_spinor<double, float>(h->g, h->lam32, h->lam64, h->p.n_v, h->st));

@@ -245,7 +245,8 @@ size_t l2_assemble_smem(int n1, int n2v, int real_size);
 // ---- coarse grid ----------------------------------------------------------------
 // classical Gram-Schmidt twice per (aggregate, chirality) on n FP64 or FP32
 // fields
-cudaError_t orthonormalise(const Geom& g, double* lam, int n, cudaStream_t st);
+// (lam32, nullable: receives the vectors in FP32)
+cudaError_t orthonormalise(const Geom& g, double* lam, float* lam32, int n, cudaStream_t st);
 cudaError_t orthonormalise(const Geom& g, float* lam, int n, cudaStream_t st);
 // b_c = R b  (coarse layout [rhs][X][2n] complex)
 template <class R>
