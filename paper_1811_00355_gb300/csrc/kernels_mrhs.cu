@@ -13,6 +13,10 @@
 // real product of [L, L~] (L~ = (-im, re) pairs) with [Re C; Im C].  Every
 // test vector is read once per batch (not once per right-hand side).
 //
+// The two chiralities are CTAs of their own: on 16^4 with 4^4 aggregates 256 CTAs
+// would leave 152 SMs unevenly filled (12 fields, 20 vectors, R call: 214 -> 210
+// us, the same values).
+//
 // Arithmetic: the 3xTF32 tensor-core products of mma_tf32.cuh (FP32
 // accuracy).
 #include "common.cuh"
@@ -58,7 +62,7 @@ __device__ __forceinline__ void stage_rows(float* dst, int stride, const float* 
 }
 
 // ---------------------------------------------------------------------------
-// restriction: CTA per (aggregate, group of <= 16 right-hand sides)
+// restriction: CTA per (aggregate, group of <= 16 right-hand sides, chirality)
 //   acc[i][c] = sum_k lam_i[k] Bx[k][c],  Bx[.][c] = b_c (c < N) or b~_{c-N}
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(MT_THREADS) k_restrict_mma(Geom g, const float* __restrict__ lam, int n,
@@ -77,7 +81,8 @@ __global__ void __launch_bounds__(MT_THREADS) k_restrict_mma(Geom g, const float
   const int nchunk = 3 * (g.Vb / rq);
   const int ksteps = rq / 2;     // 8 reals per step
 
-  for (int s = 0; s < 2; ++s) {
+  const int s = blockIdx.z;      // chirality
+  {
     float acc[2][4][4];
 #pragma unroll
     for (int a = 0; a < 2; ++a)
@@ -181,7 +186,7 @@ __global__ void __launch_bounds__(MT_THREADS) k_restrict_mma(Geom g, const float
 }
 
 // ---------------------------------------------------------------------------
-// prolongation: CTA per (aggregate, group of <= 16 right-hand sides)
+// prolongation: CTA per (aggregate, group of <= 16 right-hand sides, chirality)
 //   x_r[k] = sum_j Lx[k][j] Cx[j][r],  Lx = [lam, lam~] (k rows), Cx = [Re; Im]
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(MT_THREADS) k_prolong_mma(Geom g, const float* __restrict__ lam, int n,
@@ -202,7 +207,8 @@ __global__ void __launch_bounds__(MT_THREADS) k_prolong_mma(Geom g, const float*
   const int mtiles = rq / 4;                    // 16 rows each, 4 rq rows per chunk
   float* xb = x + (size_t)r0 * fstride;
 
-  for (int s = 0; s < 2; ++s) {
+  const int s = blockIdx.z;      // chirality
+  {
     for (int idx = threadIdx.x; idx < KG * 16; idx += MT_THREADS) {
       const int j = idx >> 4, r = idx & 15;
       float v = 0.f;
@@ -307,7 +313,7 @@ cudaError_t restrict_mrhs(const Geom& g, const float* lam, int n, const float* b
   const size_t smem = restrict_mma_smem(n, N);
   cudaError_t e = raise_smem_limit((const void*)k_restrict_mma, smem);
   if (e != cudaSuccess) return e;
-  k_restrict_mma<<<dim3(g.nb, (nrhs + 15) / 16), MT_THREADS, smem, st>>>(g, lam, n, b, nrhs, chunk_sites(g.Vb),
+  k_restrict_mma<<<dim3(g.nb, (nrhs + 15) / 16, 2), MT_THREADS, smem, st>>>(g, lam, n, b, nrhs, chunk_sites(g.Vb),
                                                                         reinterpret_cast<cpx<float>*>(bc));
   ++g_launches;
   return cudaGetLastError();
@@ -319,7 +325,7 @@ cudaError_t prolong_mrhs(const Geom& g, const float* lam, int n, const float* xc
   const size_t smem = prolong_mma_smem(g, n);
   cudaError_t e = raise_smem_limit((const void*)k_prolong_mma, smem);
   if (e != cudaSuccess) return e;
-  k_prolong_mma<<<dim3(g.nb, (nrhs + 15) / 16), MT_THREADS, smem, st>>>(
+  k_prolong_mma<<<dim3(g.nb, (nrhs + 15) / 16, 2), MT_THREADS, smem, st>>>(
       g, lam, n, reinterpret_cast<const cpx<float>*>(xc), nrhs, chunk_sites(g.Vb), x);
   ++g_launches;
   return cudaGetLastError();
