@@ -8,8 +8,8 @@
 // 8 (2n)^2 real multiply-adds per block and four right-hand sides run on the
 // FP32 pipe (64 us for 12).  So:
 //  * block products: a site's 2n x 2n blocks come through a ring of
-//    shared-memory slots (bulk copies, no CTA barrier per block); each of the 16 warps takes every 16th column
-//    and multiplies all 2n rows with all right-hand sides, lane (g, j) the row
+//    shared-memory slots (bulk copies, no CTA barrier per block); each of the 16
+//    warps takes every 16th column and multiplies all 2n rows with all right-hand sides, lane (g, j) the row
 //    pairs j, j + 8, .. and a quarter of the right-hand sides: per column
 //    UT + RQ shared-memory loads for 8 UT RQ multiply-adds.  The warps' sums
 //    meet in shared memory once per site.  (1.1 us per block: the pipes' own
@@ -22,7 +22,7 @@
 //  * the partial sums of all CTAs are FP32 pairs, four of them per warp in flight.
 // The form before (two row pairs and four right-hand sides per thread, a CTA
 // barrier per block, vectors staged before each site, passes of eight) took
-// 530 us per iteration of 12 right-hand sides there; this one 270.
+// 530 us per iteration of 12 right-hand sides there; this one 268.
 #include <algorithm>
 
 #include "cgmres.cuh"
