@@ -134,7 +134,8 @@ struct CGA {
   cpx<R>* xg;        // [NR][NE][n2]
   unsigned char* lglob;   // per-CTA local arrays when they do not fit in smem
   size_t lstride;         // bytes per CTA in lglob
-  cpx<R>* part;      // [(MAXM + 2) * NR][G]
+  cpx<R>* part;      // [slots * NR][G]
+  int slots;         // at least MAXM + 2
   unsigned* bar;
   int* iters;
   int* iters_acc;
@@ -494,8 +495,12 @@ __global__ void __launch_bounds__(TPB) k_cgmres(CGA<R> a) {
     }
     return true;
   };
-  // partial dots (r, j < kcount) of V_j[r] with wl[r]; slot = j * NR + r
-  auto partial = [&](int kcount, bool norm) {
+  // partial dots (r, j < kcount) of V_j[r] with wl[r]; slot = (s0 + j) NR + r.
+  // Other CTAs may still be gathering the reduction before: where no grid
+  // barrier lies between that gather and this call, s0 has to lead past its
+  // slots
+  auto partial = [&](int s0, int kcount, bool norm) {
+    cpx<R>* part = a.part + (size_t)s0 * NR * G;
     const int pairs = norm ? NR : kcount * NR;
     for (int pr = wid; pr < pairs; pr += NW) {
       const int j = norm ? 0 : pr / NR, r = norm ? pr : pr - (pr / NR) * NR;
@@ -512,17 +517,18 @@ __global__ void __launch_bounds__(TPB) k_cgmres(CGA<R> a) {
       re = wsum(re);
       im = wsum(im);
       if (lane == 0) {
-        a.part[(size_t)pr * G + blockIdx.x] = mk(re, im);
+        part[(size_t)pr * G + blockIdx.x] = mk(re, im);
       }
     }
   };
   // gather slot sums into dst[r][2 j] (norm: dst[r])
-  auto gather = [&](int kcount, bool norm, A* dst, int dstride) {
+  auto gather = [&](int s0, int kcount, bool norm, A* dst, int dstride) {
+    const cpx<R>* part = a.part + (size_t)s0 * NR * G;
     const int pairs = norm ? NR : kcount * NR;
     for (int pr = wid; pr < pairs; pr += NW) {
       A re = 0, im = 0;
       for (int c = lane; c < G; c += 32) {
-        const cpx<R> z = ldc(a.part + (size_t)pr * G + c);
+        const cpx<R> z = ldc(part + (size_t)pr * G + c);
         re += z.re;
         im += z.im;
       }
@@ -624,9 +630,9 @@ __global__ void __launch_bounds__(TPB) k_cgmres(CGA<R> a) {
       xl[idx] = mk(R(0), R(0));
     }
     __syncthreads();
-    partial(1, true);
+    partial(0, 1, true);
     if (!grid_barrier(a.bar, a.status, a.spin_limit)) return;
-    gather(1, true, bnorm, 1);
+    gather(0, 1, true, bnorm, 1);
     if (tx < NR) {
       bnorm[tx] = sqrt(bnorm[tx]);
       beta[tx] = bnorm[tx];
@@ -720,7 +726,7 @@ __global__ void __launch_bounds__(TPB) k_cgmres(CGA<R> a) {
           // FP32: one classical Gram-Schmidt pass whose reduction also carries
           // ||w||^2, so ||w_new||^2 = ||w||^2 - sum_j |h_j|^2 (Pythagoras); an
           // explicit norm is taken only if that difference has cancelled
-          partial(k + 1, false);
+          partial(0, k + 1, false);
           partial_norm_slot(k + 1);
           if (!grid_barrier(a.bar, a.status, a.spin_limit)) return;
           gather_dots_norm(k + 1, hc, 2 * (m + 1), hnv);
@@ -752,9 +758,9 @@ __global__ void __launch_bounds__(TPB) k_cgmres(CGA<R> a) {
           }
           __syncthreads();
           if (any_s) {
-            partial(1, true);
+            partial(k + 2, 1, true);      // (past the dots' slots, which others may still read)
             if (!grid_barrier(a.bar, a.status, a.spin_limit)) return;
-            gather(1, true, h2, 1);
+            gather(k + 2, 1, true, h2, 1);
             if (tx < NR && exn[tx]) hnv[tx] = h2[tx];
             __syncthreads();
             if (tx < NR && act[tx]) givens(tx);
@@ -782,12 +788,19 @@ __global__ void __launch_bounds__(TPB) k_cgmres(CGA<R> a) {
           }
           if (!any_act_s) break;
         } else {
-          // FP64: classical Gram-Schmidt with one re-orthogonalisation pass
+          // FP64: classical Gram-Schmidt with one re-orthogonalisation pass.
+          // The second pass's slots follow those of the first, which others
+          // may still read; where the buffer has no room for both, everyone
+          // is waited for instead (12 right-hand sides in lockstep, beyond 33
+          // basis vectors).  The norm then takes slots that neither uses.
+          const int s1 = 2 * (k + 1) <= a.slots ? k + 1 : 0;
           for (int pass = 0; pass < 2; ++pass) {
-            partial(k + 1, false);
+            const int s0 = pass == 0 ? 0 : s1;
+            if (pass == 1 && s1 == 0 && !grid_barrier(a.bar, a.status, a.spin_limit)) return;
+            partial(s0, k + 1, false);
             if (!grid_barrier(a.bar, a.status, a.spin_limit)) return;
             A* hh = pass == 0 ? hc : h2;
-            gather(k + 1, false, hh, 2 * (m + 1));
+            gather(s0, k + 1, false, hh, 2 * (m + 1));
             for (int idx = tx; idx < NR * Lo; idx += TPB) {
               const int r = idx / Lo, e = idx - r * Lo;
               if (!act[r]) continue;
@@ -809,9 +822,11 @@ __global__ void __launch_bounds__(TPB) k_cgmres(CGA<R> a) {
             __syncthreads();
           }
           // ||w||: this barrier also publishes the neighbours' w for the next odd phase
-          partial(1, true);
+          // (slot 0 is free again where the second pass has other slots)
+          const int sn = s1 ? 0 : k + 1;
+          partial(sn, 1, true);
           if (!grid_barrier(a.bar, a.status, a.spin_limit)) return;
-          gather(1, true, hnv, 1);
+          gather(sn, 1, true, hnv, 1);
           if (tx < NR && act[tx]) givens(tx);
           __syncthreads();
           for (int idx = tx; idx < NR * Lo; idx += TPB) {
@@ -870,9 +885,9 @@ __global__ void __launch_bounds__(TPB) k_cgmres(CGA<R> a) {
       }
       if (tx < NR) act[tx] = conv[tx] ? 0 : 1;
       __syncthreads();
-      partial(1, true);
+      partial(0, 1, true);
       if (!grid_barrier(a.bar, a.status, a.spin_limit)) return;
-      gather(1, true, beta, 1);
+      gather(0, 1, true, beta, 1);
       if (tx < NR && !conv[tx]) {
         beta[tx] = sqrt(beta[tx]);
         if (beta[tx] <= (A)a.tol * bnorm[tx]) conv[tx] = 1;
@@ -1171,6 +1186,8 @@ cudaError_t coarse_gmres(const Geom& g, const CoarseSolveArgs& ca, const R* b, R
   a.xg = a.to + vec;
   size_t off = al16(3 * vec * sizeof(cpx<R>));
   a.part = reinterpret_cast<cpx<R>*>(w8 + off);
+  a.slots = (int)std::min<size_t>((size_t)(MAXM + 2) * NRMAX * NE * 2 * sizeof(double) / ((size_t)ch.NR * ch.G * sizeof(cpx<R>)),
+                                  4 * MAXM);
   off += al16((size_t)(MAXM + 2) * NRMAX * NE * 2 * sizeof(double));
   a.bar = reinterpret_cast<unsigned*>(w8 + off);
   off += 256;

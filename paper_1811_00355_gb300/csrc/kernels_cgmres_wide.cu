@@ -385,10 +385,13 @@ __global__ void __launch_bounds__(TPB, 1) k_cgmres_wide(WideArgs a) {
   };
 
   // ---- Gram-Schmidt -------------------------------------------------------------
-  // sums over this CTA of <V_j[r], w[r]> for j < kcount (slot j NR + r) and, in
-  // slot kcount NR + r, ||w[r]||^2: a warp takes a right-hand side and eight
-  // vectors at a time
-  auto partial = [&](int kcount) {
+  // sums over this CTA of <V_j[r], w[r]> for j < kcount (slot (s0 + j) NR + r)
+  // and, in slot (s0 + kcount) NR + r, ||w[r]||^2: a warp takes a right-hand
+  // side and eight vectors at a time.  Other CTAs may still be gathering the
+  // reduction before: where no grid barrier lies between that gather and this
+  // call, s0 has to lead past its slots
+  auto partial = [&](int s0, int kcount) {
+    float2* part = a.part + (size_t)s0 * NR * G;
     const int groups = (kcount + 7) / 8 > 0 ? (kcount + 7) / 8 : 1;
     for (int un = wid; un < groups * NR; un += NWARP) {
       const int r = un % NR, j0 = (un / NR) * 8;
@@ -421,16 +424,17 @@ __global__ void __launch_bounds__(TPB, 1) k_cgmres_wide(WideArgs a) {
         const int q = lane >> 2;
         const float im = __shfl_down_sync(0xffffffffu, sum, 2);
         if ((lane & 3) == 0 && j0 + q < kcount)
-          a.part[(size_t)((j0 + q) * NR + r) * G + blockIdx.x] = make_float2(sum, im);
+          part[(size_t)((j0 + q) * NR + r) * G + blockIdx.x] = make_float2(sum, im);
       }
       if (j0 == 0) {
         nn2 = wsum(nn2);
-        if (lane == 0) a.part[(size_t)(kcount * NR + r) * G + blockIdx.x] = make_float2(nn2, 0.f);
+        if (lane == 0) part[(size_t)(kcount * NR + r) * G + blockIdx.x] = make_float2(nn2, 0.f);
       }
     }
   };
   // the slots' sums over all CTAs: dots to dst[r][2 j], squared norms to nrm[r]
-  auto gather = [&](int kcount, float* dst, float* nrm) {
+  auto gather = [&](int s0, int kcount, float* dst, float* nrm) {
+    const float2* part = a.part + (size_t)s0 * NR * G;
     const int pairs = (kcount + 1) * NR;
     for (int p0 = 4 * wid; p0 < pairs; p0 += 4 * NWARP) {
       float re[4] = {}, im[4] = {};
@@ -438,7 +442,7 @@ __global__ void __launch_bounds__(TPB, 1) k_cgmres_wide(WideArgs a) {
 #pragma unroll
         for (int q = 0; q < 4; ++q)
           if (p0 + q < pairs) {
-            const float2 z = __ldcg(a.part + (size_t)(p0 + q) * G + c);
+            const float2 z = __ldcg(part + (size_t)(p0 + q) * G + c);
             re[q] += z.x;
             im[q] += z.y;
           }
@@ -490,9 +494,9 @@ __global__ void __launch_bounds__(TPB, 1) k_cgmres_wide(WideArgs a) {
               xl[o] = mk(0.f, 0.f);
             }))
       return;
-    partial(0);
+    partial(0, 0);
     if (!grid_barrier(a.bar, a.status, a.spin_limit)) return;
-    gather(0, hc, bnorm);
+    gather(0, 0, hc, bnorm);
     if (tx < NR) {
       bnorm[tx] = sqrtf(bnorm[tx]);
       beta[tx] = bnorm[tx];
@@ -588,9 +592,9 @@ __global__ void __launch_bounds__(TPB, 1) k_cgmres_wide(WideArgs a) {
         // one classical Gram-Schmidt pass whose reduction also carries ||w||^2,
         // so ||w_new||^2 = ||w||^2 - sum_j |h_j|^2 (Pythagoras); an explicit
         // norm is taken only if that difference has cancelled
-        partial(k + 1);
+        partial(0, k + 1);
         if (!grid_barrier(a.bar, a.status, a.spin_limit)) return;
-        gather(k + 1, hc, hnv);
+        gather(0, k + 1, hc, hnv);
         if (tx < NR) {
           const float* hr = hc + (size_t)tx * 2 * (m + 1);
           float s2 = hnv[tx];
@@ -623,9 +627,9 @@ __global__ void __launch_bounds__(TPB, 1) k_cgmres_wide(WideArgs a) {
         __syncthreads();
         const int any_explicit = any_s;
         if (any_explicit) {
-          partial(0);
+          partial(k + 2, 0);       // (past the dots' slots, which others may still read)
           if (!grid_barrier(a.bar, a.status, a.spin_limit)) return;
-          gather(0, hc, h2);
+          gather(k + 2, 0, hc, h2);
           if (tx < NR && exn[tx]) hnv[tx] = h2[tx];
           __syncthreads();
         } else {
@@ -696,9 +700,9 @@ __global__ void __launch_bounds__(TPB, 1) k_cgmres_wide(WideArgs a) {
       }
       if (tx < NR) act[tx] = conv[tx] ? 0 : 1;
       __syncthreads();
-      partial(0);
+      partial(0, 0);
       if (!grid_barrier(a.bar, a.status, a.spin_limit)) return;
-      gather(0, hc, beta);
+      gather(0, 0, hc, beta);
       if (tx < NR && !conv[tx]) {
         beta[tx] = sqrtf(beta[tx]);
         if (beta[tx] <= a.tol * bnorm[tx]) conv[tx] = 1;
