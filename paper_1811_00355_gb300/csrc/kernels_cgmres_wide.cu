@@ -149,6 +149,7 @@ __global__ void __launch_bounds__(TPB, 1) k_cgmres_wide(WideArgs a) {
   float* Rf = reinterpret_cast<float*>(lbase + al16((size_t)(m + 4) * NR * L * 8));   // [NR][m(m+1)] packed columns
   __shared__ int any_s, any_act_s, exn[NR];
   __shared__ __align__(8) uint64_t full[RING_MAX], empty[RING_MAX];   // a slot's block has landed / is done with
+  __shared__ signed char sent[RING_MAX];      // the phase parity of `full` that a slot's last copy completes; -1: no copy yet
 
   const int G = gridDim.x, tx = threadIdx.x, wid = tx >> 5, lane = tx & 31;
   const int gq = lane >> 3, jq = lane & 7;          // right-hand-side quarter, row-pair slot
@@ -168,6 +169,7 @@ __global__ void __launch_bounds__(TPB, 1) k_cgmres_wide(WideArgs a) {
     for (unsigned q = 0; q < RING; ++q) {
       mbar_init(&full[q], 1);
       mbar_init(&empty[q], NWARP);
+      sent[q] = -1;
     }
     mbar_fence_init();
   }
@@ -200,7 +202,9 @@ __global__ void __launch_bounds__(TPB, 1) k_cgmres_wide(WideArgs a) {
     const unsigned nd = kind == K_EVEN ? 9 : 8;
     return a.Dc + ((size_t)a.g.ceven[lo + i / nd] * 9 + (9 - nd) + i % nd) * nn;
   };
-  auto copy = [&](int kind, unsigned base, unsigned q, unsigned i) {
+  // (parity: that of block i's use of slot q)
+  auto copy = [&](int kind, unsigned base, unsigned q, unsigned parity, unsigned i) {
+    sent[q] = (signed char)parity;
     mbar_expect_tx(&full[q], nn * 8);
     bulk_g2s(ringbuf + (size_t)q * nn, blk(kind, i - base), nn * 8, &full[q]);
   };
@@ -209,8 +213,28 @@ __global__ void __launch_bounds__(TPB, 1) k_cgmres_wide(WideArgs a) {
   auto prime = [&](int kind) {
     const unsigned nd = kind == K_INV ? 1 : kind == K_EVEN ? 9 : 8, n = min(RING, nown * nd);
     if (tx == 0)
-      for (unsigned i = primed; i < n; ++i) copy(kind, used, (slot + i) % RING, used + i);
+      for (unsigned i = primed; i < n; ++i) {
+        const unsigned at = slot + i;         // (at most RING - 1 past the last slot)
+        copy(kind, used, at % RING, at < RING ? turn : turn ^ 1u, used + i);
+      }
     primed = n;
+  };
+  // before the CTA leaves early (all threads past a CTA barrier): every copy
+  // that was sent has landed, each wait bounded
+  auto drain = [&]() {
+    if (tx == 0)
+      for (unsigned q = 0; q < RING; ++q)
+        if (sent[q] >= 0) mbar_wait_bounded(&full[q], (unsigned)sent[q], MBAR_POLL_LIMIT);
+  };
+  // the grid barriers; false (copies on their way waited for) when one gives up
+  auto others = [&]() -> bool {
+    if (grid_wait(a.bar, a.status, a.spin_limit)) return true;
+    drain();
+    return false;
+  };
+  auto meet = [&]() -> bool {
+    grid_arrive(a.bar);
+    return others();
   };
   // vectors that block d0 + t of site si multiplies, into buffer `buf`:
   // src(si, t, r) is the address of n2 entries (16-byte pieces)
@@ -256,7 +280,7 @@ __global__ void __launch_bounds__(TPB, 1) k_cgmres_wide(WideArgs a) {
           for (int q = 0; q < RQ; ++q) acc[u][e][q] = mk(0.f, 0.f);
       for (int t = 0; t < nd; ++t) {
         const unsigned b = base + (unsigned)(si * nd + t);
-        ok = mbar_wait_bounded(&full[slot], turn, a.spin_limit) && ok;
+        if (ok) ok = mbar_wait_bounded(&full[slot], turn, a.spin_limit);
         // columns wid + 16 i: the lane's row pairs and right-hand sides
         const float4 *M = reinterpret_cast<const float4*>(ringbuf + (size_t)slot * nn) + wid * np + jq, *Ml = M + last;
         const cpx<float>* vt = sv + (size_t)t * NR * svs + wid;
@@ -279,13 +303,15 @@ __global__ void __launch_bounds__(TPB, 1) k_cgmres_wide(WideArgs a) {
 #pragma unroll
         for (int i = 0; i + 1 < UT; ++i) column(i);
         if (UT - 1 < ncol) column(UT - 1);
-        __syncwarp();
-        if (lane == 0) {
+        // (a warp that has given up neither frees a slot nor fills one: a
+        // slot's copies follow one another, each after the one before landed)
+        ok = __all_sync(0xffffffffu, ok);
+        if (lane == 0 && ok) {
           mbar_arrive(&empty[slot]);
           if (wid == (int)(b % NWARP) && b > base && b - 1 + RING < end) {
-            const unsigned before = slot ? slot - 1 : RING - 1;
-            ok = mbar_wait_bounded(&empty[before], slot ? turn : turn ^ 1u, a.spin_limit) && ok;
-            copy(kind, base, before, b - 1 + RING);
+            const unsigned before = slot ? slot - 1 : RING - 1, p = slot ? turn : turn ^ 1u;
+            ok = mbar_wait_bounded(&empty[before], p, a.spin_limit);
+            if (ok) copy(kind, base, before, p ^ 1u, b - 1 + RING);
           }
         }
         if (++slot == RING) {
@@ -294,12 +320,8 @@ __global__ void __launch_bounds__(TPB, 1) k_cgmres_wide(WideArgs a) {
         }
       }
       if (__syncthreads_or(!ok)) {
-        if (tx == 0) {
-          atomicExch(a.status, 6);
-          // all that may be on their way: the next RING blocks (each wait bounded)
-          for (unsigned i = 0; i < RING && base + (unsigned)((si + 1) * nd) + i < end; ++i)
-            mbar_wait_bounded(&full[(slot + i) % RING], slot + i < RING ? turn : turn ^ 1u, MBAR_POLL_LIMIT);
-        }
+        if (tx == 0) atomicExch(a.status, 6);
+        drain();
         asm volatile("cp.async.wait_group 0;" ::: "memory");
         return false;
       }
@@ -481,7 +503,7 @@ __global__ void __launch_bounds__(TPB, 1) k_cgmres_wide(WideArgs a) {
         }))
       return;
     prime(K_EVEN_HOPS);
-    if (!grid_barrier(a.bar, a.status, a.spin_limit)) return;
+    if (!meet()) return;
     // rhs_e = b_e - D_eo to; x_e = 0; w = rhs_e
     if (!products(
             K_EVEN_HOPS, [&](int si, int t, int r) { return a.to + r * vstr + nbo[(a.per + si) * 8 + t]; },
@@ -495,7 +517,7 @@ __global__ void __launch_bounds__(TPB, 1) k_cgmres_wide(WideArgs a) {
             }))
       return;
     partial(0, 0);
-    if (!grid_barrier(a.bar, a.status, a.spin_limit)) return;
+    if (!meet()) return;
     gather(0, 0, hc, bnorm);
     if (tx < NR) {
       bnorm[tx] = sqrtf(bnorm[tx]);
@@ -530,7 +552,7 @@ __global__ void __launch_bounds__(TPB, 1) k_cgmres_wide(WideArgs a) {
         Vk(0, r)[e] = scl[r] * v;
         a.wg[r * vstr + (size_t)lo * n2 + e] = v;
       }
-      if (!grid_barrier(a.bar, a.status, a.spin_limit)) return;
+      if (!meet()) return;
       for (int k = 0; k < m; ++k) {
         // w = S V_k: odd phase from the neighbours' unnormalised w (scale 1/h)
         if (!phase_odd(a.wg)) return;
@@ -540,7 +562,7 @@ __global__ void __launch_bounds__(TPB, 1) k_cgmres_wide(WideArgs a) {
           const float4 v = reinterpret_cast<const float4*>(Vk(k, r))[e];
           reinterpret_cast<float4*>(wl + (size_t)r * L)[e] = make_float4(-v.x, -v.y, -v.z, -v.w);
         });
-        if (!grid_barrier(a.bar, a.status, a.spin_limit)) return;
+        if (!meet()) return;
         if (!phase_even(wl, wl)) return;
         prime(K_ODD);
         // Givens rotation of right-hand side r's new Hessenberg column (one
@@ -593,7 +615,7 @@ __global__ void __launch_bounds__(TPB, 1) k_cgmres_wide(WideArgs a) {
         // so ||w_new||^2 = ||w||^2 - sum_j |h_j|^2 (Pythagoras); an explicit
         // norm is taken only if that difference has cancelled
         partial(0, k + 1);
-        if (!grid_barrier(a.bar, a.status, a.spin_limit)) return;
+        if (!meet()) return;
         gather(0, k + 1, hc, hnv);
         if (tx < NR) {
           const float* hr = hc + (size_t)tx * 2 * (m + 1);
@@ -628,7 +650,7 @@ __global__ void __launch_bounds__(TPB, 1) k_cgmres_wide(WideArgs a) {
         const int any_explicit = any_s;
         if (any_explicit) {
           partial(k + 2, 0);       // (past the dots' slots, which others may still read)
-          if (!grid_barrier(a.bar, a.status, a.spin_limit)) return;
+          if (!meet()) return;
           gather(k + 2, 0, hc, h2);
           if (tx < NR && exn[tx]) hnv[tx] = h2[tx];
           __syncthreads();
@@ -650,7 +672,7 @@ __global__ void __launch_bounds__(TPB, 1) k_cgmres_wide(WideArgs a) {
           any_act_s = any;
         }
         if (!any_explicit) {
-          if (!grid_wait(a.bar, a.status, a.spin_limit)) return;
+          if (!others()) return;
         } else {
           __syncthreads();
         }
@@ -688,11 +710,11 @@ __global__ void __launch_bounds__(TPB, 1) k_cgmres_wide(WideArgs a) {
         wl[(size_t)r * L + e] = mk(-s.re, -s.im);      // the self block's vector below
       }
       if (tx < NR) scl[tx] = 1.f;
-      if (!grid_barrier(a.bar, a.status, a.spin_limit)) return;
+      if (!meet()) return;
       // true residual w = rhs_e - S x_e
       if (!phase_odd(a.xg)) return;
       prime(K_EVEN);
-      if (!grid_barrier(a.bar, a.status, a.spin_limit)) return;
+      if (!meet()) return;
       if (!phase_even(wl, wl)) return;
       for (int idx = tx; idx < NR * Lo; idx += TPB) {
         const int r = idx / Lo, e = idx - r * Lo;
@@ -701,7 +723,7 @@ __global__ void __launch_bounds__(TPB, 1) k_cgmres_wide(WideArgs a) {
       if (tx < NR) act[tx] = conv[tx] ? 0 : 1;
       __syncthreads();
       partial(0, 0);
-      if (!grid_barrier(a.bar, a.status, a.spin_limit)) return;
+      if (!meet()) return;
       gather(0, 0, hc, beta);
       if (tx < NR && !conv[tx]) {
         beta[tx] = sqrtf(beta[tx]);
@@ -717,7 +739,7 @@ __global__ void __launch_bounds__(TPB, 1) k_cgmres_wide(WideArgs a) {
       if (r < nr) xx[(size_t)r * NX * n2 + (size_t)a.g.ceven[lo + e / n2] * n2 + e % n2] = v;
     }
     if (tx < NR) scl[tx] = 1.f;
-    if (!grid_barrier(a.bar, a.status, a.spin_limit)) return;
+    if (!meet()) return;
     auto xo = [&](int si, int r, int row) { return xx + (size_t)r * NX * n2 + (size_t)a.g.codd[lo + si] * n2 + row; };
     if (!phase_inv(bb, nr, [&](int si, int r, int row, cpx<float> s) {
           if (r < nr) *xo(si, r, row) = s;
@@ -733,7 +755,7 @@ __global__ void __launch_bounds__(TPB, 1) k_cgmres_wide(WideArgs a) {
       if (a.iters) a.iters[r0 + tx] = tot[tx];
       if (a.iters_acc) atomicAdd(a.iters_acc, tot[tx]);
     }
-    if (!grid_barrier(a.bar, a.status, a.spin_limit)) return;
+    if (!meet()) return;
   }
 }
 
