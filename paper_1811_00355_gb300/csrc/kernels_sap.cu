@@ -944,8 +944,10 @@ __global__ void __launch_bounds__(VB, 256 / VB) k_sap_block(SapArgs a) {
             sre += q.x; sim += q.y; spp += q.z;
           }
           if (spp > 0.f) {
-            const float inv = 1.f / spp;
-            const f2 al = mk(sre * inv, sim * inv);
+            // (residuals down to 1e-21 a component: the reciprocal of a sum
+            // below 2^-128 is infinite, so small sums are scaled first)
+            const float up = spp < 0x1p-100f ? 0x1p64f : 1.f, inv = 1.f / (spp * up);
+            const f2 al = mk(sre * up * inv, sim * up * inv);
             if (t == 0) alpha = make_float2(al.re, al.im);
 #pragma unroll
             for (int u = 0; u < 6; ++u) {

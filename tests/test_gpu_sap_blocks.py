@@ -46,3 +46,30 @@ def test_cycles_and_iterations(n_sap, mr):
         assert_close(got[k], smoother(cfg).apply(t(x[k]), n_sap, mr).numpy(), 2e-5)
     assert not np.any(s.sap(np.zeros_like(x), 1))  # <p,p> = 0: the step is skipped
     s.close()
+
+
+@pytest.mark.parametrize("cfg", [((8, 8, 8, 8), (4, 4, 4, 4), 0.3, -0.2, 1.0, 1, 0),
+                                 ((4, 4, 8, 64), (2, 2, 4, 4), 0.3, 1.0, 1.0, 1, 0)])
+@pytest.mark.parametrize("prec", [1, 2, 3])
+def test_residuals_near_underflow(cfg, prec):
+    """Fields so small that <p,p> of a block becomes subnormal, and point
+    sources whose far blocks do: finite everywhere.  Squares of components
+    underflow below 4e-23, so at 1e-17 the residuals that the sums still
+    resolve are 4e-6 of the field and the bounds hold; at 1e-19 the smoother
+    still brings the error below that of x = 0."""
+    L = cfg[0]
+    s, ref = make(cfg, prec), smoother(cfg)
+    v = syn.gaussian_spinors(1, L, 12)[0]
+    point = np.zeros_like(v)
+    point[0, 0, 0] = 1.0
+    y, yp = ref.apply(t(v), 4, 4).numpy(), ref.apply(t(point), 4, 4).numpy()
+    tol = 2e-5 if prec == 1 else 2e-2
+    for b, want, scales in ((v, y, (1e-15, 1e-17, 1e-19, 1e-21, 1e-23)), (point, yp, (1.0, 1e-10, 1e-15))):
+        got = s.sap(np.stack([k * b for k in scales]), prec)
+        for k, g in zip(scales, got):
+            assert np.isfinite(g).all(), k
+            if k >= 1e-17:
+                assert_close(g, k * want, tol, f"scale {k}")
+            elif k >= 1e-19:
+                assert np.linalg.norm(g - k * want) < np.linalg.norm(k * want)
+    s.close()
