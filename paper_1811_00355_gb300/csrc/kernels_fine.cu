@@ -279,8 +279,9 @@ __device__ __forceinline__ void pack6(const c64 (&m)[6][6], double* P) {
 }
 
 // ---------------------------------------------------------------------------
-// gauge import: two rows of each link in FP32, with the third row rebuilt from
-// them in FP64, + SU(3) check
+// gauge import: two rows of each link in FP32, the whole link as given in FP64
+// (the clover term and D of links that are SU(3) only to the accepted 1e-9 are
+// those of these links), + SU(3) check
 // ---------------------------------------------------------------------------
 __global__ void k_import_gauge(Geom g, const double* __restrict__ lex, double* __restrict__ g64,
                                float* __restrict__ g32, unsigned long long* dev_dev) {
@@ -303,12 +304,9 @@ __global__ void k_import_gauge(Geom g, const double* __restrict__ lex, double* _
               U.a[0][2] * (U.a[1][0] * U.a[2][1] - U.a[1][1] * U.a[2][0]);
     worst = fmax(worst, sqrt(norm2(det - mk(1.0, 0.0))));
     if (!(worst == worst)) worst = 1e300;   // NaN
-    Link<double> T;
-    for (int k = 0; k < 6; ++k) T.m[k / 3][k % 3] = U.a[k / 3][k % 3];
-    complete_link(T);
     for (int k = 0; k < 9; ++k) {
-      v64[mu * LINK64_NR + 2 * k] = T.m[k / 3][k % 3].re;
-      v64[mu * LINK64_NR + 2 * k + 1] = T.m[k / 3][k % 3].im;
+      v64[mu * LINK64_NR + 2 * k] = U.a[k / 3][k % 3].re;
+      v64[mu * LINK64_NR + 2 * k + 1] = U.a[k / 3][k % 3].im;
     }
   }
   store_site<double, GAUGE64_NR>(g64, d, g.Vb, v64);
