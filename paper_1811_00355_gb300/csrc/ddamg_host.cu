@@ -597,16 +597,22 @@ ddamg_status import_fields(ddamg_ctx* h, const double* src, int on_device, int n
   CK(pack_spinor<R>(h->g, lex, dst, nf, h->st));
   return DDAMG_OK;
 }
-// lexicographic FP64 links (72 doubles a site: staged like three fields when
-// they come from the host)
+// lexicographic FP64 links, 72 doubles a site.  Links from the host go through
+// the staging buffer in as many pieces as its present size needs: one field of
+// it (24 doubles a site) is all that a handle's first links ask for beyond
+// the links themselves
 ddamg_status import_links(ddamg_ctx* h, const double* src, int on_device) {
-  const double* lex = src;
-  if (!on_device) {
-    TRY(need_lexbuf(h, 3));
-    CK(cudaMemcpyAsync(h->lexbuf, src, 3 * h->V24 * sizeof(double), cudaMemcpyHostToDevice, h->st));
-    lex = h->lexbuf;
+  if (on_device) {
+    CK(import_gauge(h->g, src, 0, h->g.V, h->g64, h->g32, h->d_dev, h->st));
+    return DDAMG_OK;
   }
-  CK(import_gauge(h->g, lex, h->g64, h->g32, h->d_dev, h->st));
+  TRY(need_lexbuf(h, 1));
+  const size_t room = h->lexbuf_fields * h->V24 / 72;
+  for (size_t x0 = 0; x0 < (size_t)h->g.V; x0 += room) {
+    const size_t n = std::min(room, (size_t)h->g.V - x0);
+    CK(cudaMemcpyAsync(h->lexbuf, src + x0 * 72, n * 72 * sizeof(double), cudaMemcpyHostToDevice, h->st));
+    CK(import_gauge(h->g, h->lexbuf, (int)x0, (int)n, h->g64, h->g32, h->d_dev, h->st));
+  }
   return DDAMG_OK;
 }
 template <class R>

@@ -75,10 +75,11 @@ template <class RD, class RS>
 cudaError_t convert_spinor(const Geom& g, const RS* src, RD* dst, int nf, cudaStream_t st);
 
 // ---- gauge and clover -------------------------------------------------------
-// lexicographic FP64 links into the device layouts (as given in FP64, two rows
-// in FP32); the largest deviation from SU(3) (|U U^H - 1|, |det U - 1|) is max-reduced into
-// *dev_dev (as ordered bits of a non-negative double)
-cudaError_t import_gauge(const Geom& g, const double* lex, double* g64, float* g32,
+// lexicographic FP64 links of sites first .. first + sites - 1 (lex: those of
+// site `first`) into the device layouts (as given in FP64, two rows in FP32);
+// the largest deviation from SU(3) (|U U^H - 1|, |det U - 1|) is max-reduced
+// into *dev_dev (as ordered bits of a non-negative double)
+cudaError_t import_gauge(const Geom& g, const double* lex, int first, int sites, double* g64, float* g32,
                          unsigned long long* dev_dev, cudaStream_t st);
 // A = (4 + m0) + C and A^-1, packed, in FP64 and FP32 device layouts
 cudaError_t build_clover(const Geom& g, const double* g64, double m0, double csw,

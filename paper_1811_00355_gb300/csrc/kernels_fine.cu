@@ -283,11 +283,12 @@ __device__ __forceinline__ void pack6(const c64 (&m)[6][6], double* P) {
 // (the clover term and D of links that are SU(3) only to the accepted 1e-9 are
 // those of these links), + SU(3) check
 // ---------------------------------------------------------------------------
-__global__ void k_import_gauge(Geom g, const double* __restrict__ lex, double* __restrict__ g64,
+__global__ void k_import_gauge(Geom g, const double* __restrict__ lex, int first, int sites, double* __restrict__ g64,
                                float* __restrict__ g32, unsigned long long* dev_dev) {
   int d = blockIdx.x * blockDim.x + threadIdx.x;
   if (d >= g.V) return;
-  int x = g.lex_of_dev[d];
+  int x = g.lex_of_dev[d] - first;
+  if (x < 0 || x >= sites) return;
   double v64[GAUGE64_NR];
   double worst = 0.0;
   for (int mu = 0; mu < 4; ++mu) {
@@ -835,9 +836,9 @@ cudaError_t convert_spinor(const Geom& g, const RS* src, RD* dst, int nf, cudaSt
 template cudaError_t convert_spinor<float, double>(const Geom&, const double*, float*, int, cudaStream_t);
 template cudaError_t convert_spinor<double, float>(const Geom&, const float*, double*, int, cudaStream_t);
 
-cudaError_t import_gauge(const Geom& g, const double* lex, double* g64, float* g32,
+cudaError_t import_gauge(const Geom& g, const double* lex, int first, int sites, double* g64, float* g32,
                          unsigned long long* dev_dev, cudaStream_t st) {
-  k_import_gauge<<<nblk(g.V, TPB), TPB, 0, st>>>(g, lex, g64, g32, dev_dev);
+  k_import_gauge<<<nblk(g.V, TPB), TPB, 0, st>>>(g, lex, first, sites, g64, g32, dev_dev);
   ++g_launches;
   return cudaGetLastError();
 }
