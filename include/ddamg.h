@@ -358,7 +358,8 @@ DDAMG_API ddamg_status ddamg_get_coarse_plan(ddamg_handle h, int nrhs, ddamg_coa
  * problem, the variants' mean times in microseconds and the choice.
  * Variants so far: the Wilson-clover D with one thread per site (0) or four
  * threads per site, one hop direction each (1), in FP32 and in BF16/FP16
- * storage; the FP32
+ * storage (FP32: the solver's operator, and under problems ending in "call"
+ * ddamg_apply_D with its output in the exchange layout); the FP32
  * Schwarz sweep with the block's links and clover blocks in registers and the
  * residual carried between sweeps (0) or by the general kernel (1) ("SAP
  * fp32"; the half-storage sweep has one form); the

@@ -2783,22 +2783,29 @@ ddamg_status ddamg_apply_D(ddamg_handle h, int prec, int nrhs, const double* in,
       TRY(need_tmp(h, nrhs, 6));
       TRY(import_fields<R>(h, in, on_device, nrhs, (R*)h->tmp[0]));
     }
-    int v = 0;
-    if constexpr (sizeof(R) == 4) TRY(dslash32_variant(h, (const float*)h->tmp[0], (float*)h->tmp[1], nrhs, &v));
-    if (v == 1) {
-      TRY(op_dslash<R>(h, DSLASH_D, (R*)h->tmp[0], nullptr, (R*)h->tmp[1], nrhs));
-      return export_fields<R>(h, (R*)h->tmp[1], nrhs, out, on_device);
-    }
     double* lex = out;
     if (!on_device) {
       TRY(need_lexbuf(h, nrhs));
       lex = h->lexbuf;
     }
-    addf(h, (double)nrhs * h->g.V * F_D);
-    CK(timed(h, 0, [&] {
+    // FP32: one thread per site that writes the exchange layout itself (0), or
+    // four threads per site and then the unpacking pass (1).  Measured as they
+    // are run here: the bare operators (tuned under their own key for the
+    // solver) leave that pass out.
+    auto run = [&](int var) -> cudaError_t {
+      if constexpr (sizeof(R) == 4)
+        if (var == 1) {
+          const cudaError_t e = dslash4<float>(h->g, h->tmp[0], nullptr, h->tmp[1], nullptr, h->g32, h->A32, nrhs, h->st);
+          return e != cudaSuccess ? e : unpack_spinor<float>(h->g, (const float*)h->tmp[1], lex, nrhs, h->st);
+        }
       return dslash_lex<R>(h->g, lex_in ? (const R*)in : (const R*)h->tmp[0], lex_in, lex, gauge_of<R>(h),
                            clov_of<R>(h, false), nrhs, h->st);
-    }));
+    };
+    int v = 0;
+    if (sizeof(R) == 4 && h->g.V % 8 == 0)
+      TRY(tuned(h, "D fp32", lattice_key(h, "fp32", nrhs) + " call", 2, run, &v));
+    addf(h, (double)nrhs * h->g.V * F_D);
+    CK(timed(h, 0, [&] { return run(v); }));
     if (!on_device)
       CK(cudaMemcpyAsync(out, lex, nrhs * h->V24 * sizeof(double), cudaMemcpyDeviceToHost, h->st));
     CK(cudaStreamSynchronize(h->st));

@@ -51,3 +51,32 @@ def test_fp64_D_in_place_and_unaligned():
             got = buf[out_at:out_at + n].cpu().numpy().view(np.complex128).reshape(x.shape)
             assert_close(got, ref, tol, f"precision {prec} in {shift} out {out_at}")
     s.close()
+
+
+def test_fp32_D_call_is_measured_as_it_runs():
+    """The FP32 D call records its own choice, made of both whole calls (the
+    four-threads form needs a pass to unpack, the other does not), and either
+    form on host, device and overlapping buffers gives the oracle's result."""
+    import ctypes as C
+    import paper_1811_00355_gb300 as P
+    L, block = (8, 4, 4, 12), (4, 2, 2, 6)
+    x = syn.gaussian_spinors(3, L, 18)
+    ref = oracle_op(L, 0.3, 4, -0.2, 1.0).apply(t(x)).numpy()
+    s = make((L, block, 0.3, -0.2, 1.0, 1, 4), 1)
+    for variant in (-1, 0, 1):
+        P.pin_variant("D fp32", variant)
+        try:
+            assert_close(s.apply_D(x, 1), ref, TOL32, f"host, variant {variant}")
+            buf = torch.from_numpy(x).cuda()
+            torch.cuda.synchronize()
+            assert_close(s.apply_D(buf, 1).cpu().numpy(), ref, TOL32, f"device, variant {variant}")
+            p = C.c_void_p(buf.data_ptr())
+            assert s.lib.ddamg_apply_D(s.h, 1, 3, p, p, 1) == 0
+            assert_close(buf.cpu().numpy(), ref, TOL32, f"in place, variant {variant}")
+        finally:
+            P.pin_variant("D fp32", -1)
+    rec = [r for r in P.tuning() if r["kernel"] == "D fp32" and r["problem"].startswith("8x4x4x12/4x2x2x6")
+           and r["problem"].endswith("nrhs 3 call")]
+    assert len(rec) == 1 and len(rec[0]["us"]) == 2, P.tuning()
+    assert rec[0]["us"][rec[0]["best"]] == min(rec[0]["us"])
+    s.close()
