@@ -794,7 +794,11 @@ __global__ void __launch_bounds__(VB, 256 / VB) k_sap_block(SapArgs a) {
     if (x_phase >= 0) mbar_wait_bounded(&bar_x, x_phase & 1, MBAR_POLL_LIMIT);
     return false;
   };
-  if (!landed(&bar_ops, 0, -1, -1)) return;
+  if (!landed(&bar_ops, 0, -1, -1)) {
+    // not before the sweep before: the next one waits for this grid only
+    grid_dependency_wait();
+    return;
+  }
   Link<float> U[4];
   float P[72];
   Ops<S>::links(sl, Vb, t, U);

@@ -73,3 +73,28 @@ def test_residuals_near_underflow(cfg, prec):
             elif k >= 1e-19:
                 assert np.linalg.norm(g - k * want) < np.linalg.norm(k * want)
     s.close()
+
+
+@pytest.mark.parametrize("L,block", [SHAPES[0], SHAPES[3], SHAPES[6]])
+def test_bounded_waits(L, block):
+    """Sweeps whose waits for staged data give up (wait limits from no poll to
+    many): DDAMG_ETIMEOUT or the result, and with the default limits the same
+    handle returns the same bits as before."""
+    import paper_1811_00355_gb300 as P
+    s = make((L, block, 0.3, -0.2, 1.0, 1, 0), 1)
+    x = syn.gaussian_spinors(3, L, 19)
+    P.pin_variant("SAP fp32", 0)
+    try:
+        ref = s.sap(x, 1)
+        for polls in (0, 0, 1, 2, 4, 8, 16):
+            s.set_wait_limit(polls)
+            try:
+                s.sap(x, 1)
+                assert polls > 0
+            except P.DDAMGError as e:
+                assert e.status == 6, e
+            s.set_wait_limit(-1)
+            assert np.array_equal(s.sap(x, 1), ref), polls
+    finally:
+        P.pin_variant("SAP fp32", -1)
+        s.close()
