@@ -1016,6 +1016,19 @@ Choice choose(const Geom& g, int n2, int m, int nrhs, bool wide) {
 template <class R>
 Choice choose_uncached(int dev, const Geom& g, int n2, int m, int nrhs, bool wide) {
   if (sizeof(R) == 4 && wide) {
+    // From five right-hand sides on the wide kernel is the faster one (us per
+    // iteration, wide against narrow; 4^4 coarse sites, n_v 20: five 31.8 / 43.1,
+    // eight 31.8 / 34.7, twelve 37.7 / 44.2, thirteen 73.2 / 84.7; 2^4 sites, n_v 20:
+    // 30.6 / 40.6, 30.7 / 33.3, 36.5 / 42.4, 70.7 / 81.6; 6^3 x 12 sites, n_v 24:
+    // 183 / 413, 189 / 293, 249 / 362, 470 / 698), with one exception: eight
+    // with 32-row blocks resident, one even site per CTA, where the narrow
+    // kernel's row pairs, slices, directions and column chunks come to its 512
+    // threads exactly (4^4 sites 28.7 / 25.7, 2^4 26.7 / 24.2; with n_v 17
+    // 31.4 / 34.1, with two sites per CTA 40.1 / 50.8).
+    if (nrhs == 8 && n2 == 32) {
+      const Choice c = choose_uncached<R>(dev, g, n2, m, nrhs, false);
+      if (c.NR == 8 && c.resident) return c;
+    }
     const WideChoice w = cgmres_wide_choose(dev, g, n2, m, nrhs);
     if (w.NR) {
       Choice c{};

@@ -62,3 +62,30 @@ def test_all_zero():
     Dc = syn.coarse_stencil(32, 40, 9, DIAG, HOP)
     x, its = _solve((2, 2, 2, 4), 20, 30, 300, Dc, np.zeros((6, 32, 40), complex), 5e-2)
     assert not its.any() and not x.any()
+
+
+@pytest.mark.parametrize("cL,resident", [((2, 2, 2, 2), 1), ((4, 4, 4, 4), 1), ((4, 4, 4, 6), 0)])
+def test_eight_with_32_row_blocks(cL, resident):
+    """Eight right-hand sides, n_v 16: resident blocks where a CTA owns one
+    site, else the ring."""
+    import paper_1811_00355_gb300 as P
+    geom = Geometry(cL)
+    Dc = syn.coarse_stencil(geom.V, 32, 10, DIAG, HOP)
+    cop = CoarseOperator(torch.from_numpy(Dc), geom)
+    gen = np.random.default_rng(74)
+    bc = gen.standard_normal((8, geom.V, 32)) + 1j * gen.standard_normal((8, geom.V, 32))
+    L = tuple(2 * v for v in cL)
+    s = P.DDAMG(P.default_params(L=L, sap_block=(2, 2, 2, 2), n_v=16, precision=P.FP32, coarse_max_iter=6),
+                syn.unit_gauge(L))
+    try:
+        s.set_coarse_op(Dc)
+        plan = s.coarse_plan(8)
+        assert plan["rhs_per_pass"] == 8 and plan["resident_blocks"] == resident, plan
+        assert plan["block_ring"] == 1 - resident, plan
+        x, its = s.coarse_solve(bc, 1e-30, P.FP32)
+        assert np.all(its == 6)
+        for r in range(8):
+            xr, _ = cop.solve(torch.from_numpy(bc[r]), 1e-30, 30, 6)
+            assert_close(x[r], xr.numpy(), 1e-4, f"rhs {r}")
+    finally:
+        s.close()
