@@ -80,3 +80,31 @@ def test_fp64_more_vectors_than_the_buffer_holds_twice():
             assert_close(x[r], ref.numpy(), 1e-10, f"rhs {r}")
     finally:
         s.close()
+
+
+@pytest.mark.parametrize("nrhs,restart", [(8, 8), (12, 4)])
+def test_narrow_ring_at_full_width(nrhs, restart):
+    """The narrow kernel's block ring with 8 and 12 right-hand sides in
+    lockstep, two sites per CTA, which the no-allocation call alone reaches:
+    the oracle's Krylov iterate after six iterations (bound 1e-4 as in
+    test_gpu_coarse_plans)."""
+    import paper_1811_00355_gb300 as P
+    fine = (8, 8, 8, 16)
+    geom = Geometry((4, 4, 4, 8))
+    Dc = syn.coarse_stencil(geom.V, 32, 23, 1.0, 0.21)
+    cop = CoarseOperator(torch.from_numpy(Dc), geom)
+    gen = np.random.default_rng(66)
+    bc = gen.standard_normal((nrhs, geom.V, 32)) + 1j * gen.standard_normal((nrhs, geom.V, 32))
+    s = P.DDAMG(P.default_params(L=fine, sap_block=BLOCK, n_v=16, precision=P.FP32, coarse_restart=restart,
+                                 coarse_max_iter=6), syn.unit_gauge(fine))
+    try:
+        s.set_coarse_op(Dc)
+        dev = torch.from_numpy(bc).cuda()
+        torch.cuda.synchronize()
+        x, its = s.coarse_solve_noalloc(dev, 1e-30)
+        assert np.all(its == 6), its
+        for r in range(nrhs):
+            ref, _ = cop.solve(torch.from_numpy(bc[r]), 1e-30, restart, 6)
+            assert_close(x[r].cpu().numpy(), ref.numpy(), 1e-4, f"rhs {r}")
+    finally:
+        s.close()
