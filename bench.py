@@ -45,7 +45,7 @@ L2_BYTES = 129 * 2 ** 20
 # workload, from an ncu capture of the kernel as it is now (a single-RHS
 # coarse solve); None where no capture of a single-RHS launch of the kernel
 # as it is now exists
-TRAFFIC_BYTES_PER_LAUNCH = {"sap_sweep": None, "coarse_gmres": 42_921_472 + 40_448}
+TRAFFIC_BYTES_PER_LAUNCH = {"sap_sweep": None, "coarse_gmres": 42_912_512 + 17_408}
 # stencil bandwidth lattice: 32^3 x 64 (the lattice of the batched workload),
 # far larger than L2, links tiled from an 8^4 field of the same generator
 STENCIL = dict(L=(32, 32, 32, 64), tile=(8, 8, 8, 8), block=(4, 4, 4, 4), eps=0.2, seed=3, m0=-0.3, csw=1.5,
@@ -886,7 +886,8 @@ def stencils(P, torch, stream, pk, pk_kind):
             h.enable_kernel_timing(False)
             us = 1e3 * st["dslash_ms"] / st["dslash_launches"]
             # half storage: two site norms (FP32) besides the half values;
-            # FP32 writes its output in FP64 (the exchange layout)
+            # the timed FP32 call ends with its output in FP64 (the exchange
+            # layout), in either of its variants
             byts = V * (D_REALS_PER_SITE * rs + {2: 8, 4: 24 * 4, 8: 0}[rs])
             gbs = byts / (us * 1e-6) / 1e9
             out[name] = {"us": round(us, 2), "bytes_per_launch": byts, "GB/s": round(gbs, 1),

@@ -107,7 +107,7 @@ struct ddamg_ctx {
   void* AiH[2] = {nullptr, nullptr};
   uint64_t h_gen[2] = {0, 0};
   uint64_t op_gen = 1;
-  // half spinor fields of the smoother (b, x) and of the half D (in, out),
+  // half spinor fields of the half D (in, out),
   // each with its FP32 site norms
   void* hb = nullptr;
   void* hx = nullptr;
@@ -1385,7 +1385,7 @@ ddamg_status rebuild_clover(ddamg_ctx* h, double m0, double csw) {
   return DDAMG_OK;
 }
 
-// half spinor buffers b, x (with site norms) for nf fields
+// half spinor buffers in and out of the half D (with site norms) for nf fields
 ddamg_status need_half_fields(ddamg_ctx* h, size_t nf) {
   if (h->h_fields >= nf) return DDAMG_OK;
   dfree(h, h->hb, h->h_fields * h->V24 * 2);
@@ -1403,10 +1403,6 @@ ddamg_status need_half_fields(ddamg_ctx* h, size_t nf) {
   ++h->gen;                        // captured graphs refer to the old buffers
   return DDAMG_OK;
 }
-
-
-
-
 
 ddamg_status build_coarse_op(ddamg_ctx* h) {
   if (!h->have_vectors) return fail(h, DDAMG_ESTATE, "no test vectors");

@@ -1,5 +1,6 @@
 // The coarse even-odd GMRES of kernels_cgmres.cu for many right-hand sides
-// (FP32, five or more, coarse blocks of 32 rows or more): the same method,
+// (FP32, five or more, coarse blocks of 32 to 64 rows; the rule and its one
+// exception stand at choose_uncached there): the same method,
 // CTA ownership and grid barriers, with everything else arranged for 8 or 12
 // right-hand sides in lockstep.
 //
@@ -772,7 +773,7 @@ const void* wide_fn(int NR, int n2) { return NR == 8 ? wide_kernel<8>(wide_ut(n2
 }  // namespace
 
 // NR: 12 right-hand sides in lockstep for nine or more, else 8; as many ring
-// slots (at most four) as fit beside two sites' vectors; one CTA per SM
+// slots (at most eight) as fit beside two sites' vectors; one CTA per SM
 WideChoice cgmres_wide_choose(int dev, const Geom& g, int n2, int m, int nrhs) {
   WideChoice c{};
   if (nrhs < 5 || n2 < 32 || n2 > 64) return c;

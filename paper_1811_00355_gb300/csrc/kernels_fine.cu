@@ -857,7 +857,8 @@ cudaError_t export_clover(const Geom& g, const double* dev, double* lex, cudaStr
 }
 
 // small lattices: single-warp CTAs reach all SMs (an 8^4 lattice has 32 CTAs
-// of 128 threads; the FP64 D is bound by each SM's FP64 pipe)
+// of 128 threads; the FP64 D is bound by each SM's FP64 pipe).  1216 is eight
+// CTAs for each of the 152 SMs: with fewer, smaller ones spread the sites evener
 static int dslash_threads(const Geom& g, int nrhs) {
   int threads = TPB;
   while (threads > 32 && (size_t)nblk(g.V, threads) * nrhs < 1216) threads /= 2;

@@ -1122,7 +1122,7 @@ __device__ __forceinline__ void hop_global_s(const Geom& g, const S* x, const fl
 
 // ---------------------------------------------------------------------------
 // Wilson-clover D on the whole lattice with four threads per site (the
-// thread layout of the SAP kernel): thread sub applies the two hops of
+// thread layout of the general SAP kernel): thread sub applies the two hops of
 // direction mu = sub and the three rows of its chiral clover block that it
 // owns; the hop sums are combined by warp shuffles.  A quarter of the
 // loads per thread and four times the threads of the one-thread-per-site
